@@ -343,9 +343,9 @@ int lod_root_cubes_noalloc(const lod_point_t* const* d_tiles, const uint64_t* n,
  *                   voxel levels (which need no host round trip between
  *                   them) into one CUDA graph and launches that (0: plain
  *                   launches, the default).  Ignored while profiling.
- *   vox_no_merge    1: in filtered mode the lanes of a warp whose points share
- *                   a cell do not add their colours together before updating
- *                   the table (0: they do, the default).
+ *   vox_no_merge    0 or 1, kept and without effect: the filtered voxel pass
+ *                   updates a cell by native 32-bit shared atomics, and the
+ *                   lanes of a warp that share a cell are never merged first.
  *   vox_range_cells  at most this many cells per accumulate range of the
  *                   voxel pass (1..262144; default: what shared memory
  *                   holds); smaller values only add passes. */
@@ -367,10 +367,10 @@ int lod_get_tuning(lod_tuning_t* t);
  * params; on `stream`) under candidate tunings, two builds each (the first
  * untimed), by coordinate descent from the defaults: stream_ctas_per_sm 2,
  * 3 and 4; root_depth one less and one more than the default; dense_bins_max
- * 512; vox_queue_ranges 1 (never) and 2; in filtered mode
- * vox_no_merge 1 — each knob in turn, the others held at the best so far.  Keeps the fastest with lod_set_tuning and
+ * 512; vox_queue_ranges 1 (never) and 2 — each knob in turn, the others held
+ * at the best so far.  Keeps the fastest with lod_set_tuning and
  * returns it in *best (and its build time in *best_ms when not NULL).
- * Results are freed; nothing else is kept.  Costs about 18 builds; like
+ * Results are freed; nothing else is kept.  Costs about 16 builds; like
  * lod_set_tuning it changes process-wide state, so call it while no other
  * build runs.  Returns LOD_ERR_INVALID_ARG for n == 0 or a missing pointer,
  * or the first build error (the previous tuning is then restored).  The

@@ -283,7 +283,7 @@ std::atomic<uint32_t> g_tune_queue_ranges{0};  // 0: default (4), 1: an item's r
 std::atomic<uint32_t> g_tune_range_cells{0};   // 0: what the shared memory holds
 std::atomic<uint32_t> g_tune_dense_bins{0};  // 0: kSmemBins
 std::atomic<uint32_t> g_tune_graph{0};       // 1: the voxel levels run as one CUDA graph
-std::atomic<uint32_t> g_tune_no_merge{0};    // 1: no warp merge of same-cell samples in the voxel pass
+std::atomic<uint32_t> g_tune_no_merge{0};    // kept for lod_get_tuning, without effect
 
 // Stream capture of a build's voxel levels into a CUDA graph, launched as
 // one unit on the build's stream.  The capture runs on a stream of the
@@ -1265,7 +1265,6 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
         vl.queue_ranges = q == 0 ? 4u : (q == 1 ? 0xFFFFFFFFu : q);
         vl.range_cells = g_tune_range_cells.load();
       }
-      vl.no_merge = g_tune_no_merge.load();
       if (weighted) {
         vl.wgrid = reinterpret_cast<unsigned long long*>(wbase);
         vl.wcnt = reinterpret_cast<uint32_t*>(wbase + (size_t)wctas * cells * 32);

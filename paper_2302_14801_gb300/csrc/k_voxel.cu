@@ -13,21 +13,28 @@
 //     block scan of the bitmap's population counts then stores, beside
 //     every 32-cell word of the bitmap, the rank of its first occupied
 //     cell, which numbers the item's D occupied cells 0..D-1 in cell order;
-//  2. accumulate: every sample finds its cell's rank (one 8-byte read and
-//     one population count) and updates the dense entry of that rank.
+//  2. accumulate: every sample finds its cell's rank (two reads and one
+//     population count) and updates the dense entry of that rank.
 //
 // No hashing and no probing: every lookup costs the same, D is exact before
 // anything is accumulated (so the item's staging block is reserved to the
 // record), and the voxels come out sorted by cell.  The dense entries of
-// one pass hold 5120 to 10240 cells, depending on the mode; an item with
+// one pass hold 5939 to 17817 cells, depending on the layout; an item with
 // more occupied cells takes its ranks in consecutive ranges, one accumulate
 // pass each, and may hand ranges to other SMs.  Colour sums are exact
-// integers (packed 24- or 32-bit fields while they provably cannot
-// overflow, 64-bit otherwise); the single-sample modes (minimal-hash pick,
-// first come of Section 4.2.1, random with the key of Listing 1) keep, per
-// cell, the entry {key, rgba | index << 32} of minimal key, updated by a
-// 128-bit compare-and-swap, so the picked colour travels with the winning
-// key and is never gathered from the input.
+// integers in 32-bit words (16-bit fields whose wraps are listed, 32-bit
+// sums while they provably cannot overflow, low and high words otherwise),
+// because only 32-bit shared atomic adds are native; the single-sample modes
+// (minimal-hash pick, first come of Section 4.2.1, random with the key of
+// Listing 1) keep, per cell, the smallest key by a 64-bit atomicMin, which is
+// native, and the colour of the sample that holds it.
+//
+// What bounds it: instruction issue (45 % of the slots), the shared-memory
+// data pipe (43 %, half of it the atomics' bank and address conflicts) and
+// the barriers between an item's phases.  Measured against 64-bit atomic
+// sums merged over equal lanes and 128-bit compare-and-swap picks (all levels
+// of one build, GB300): 500M indoor points filtered 11.5 -> 8.4 ms, 50M
+// aerial filtered 1.14 -> 0.74 ms, 200M indoor points picked 5.9 -> 5.5 ms.
 //
 // Every octant's voxels go to a staging area; a level scan then assigns
 // each parent one contiguous voxel range (children are consecutive in node
@@ -40,22 +47,41 @@ namespace lodk {
 
 namespace {
 
-constexpr int kSmemBytes = 224 * 1024;
-// occupancy words: 32 cells of the bitmap and the rank of their first
-// occupied cell, {word, rank} (8 bytes, one read and one population count
-// per lookup)
+// One CTA per SM with all of its shared memory.  (Two CTAs of 512 threads and
+// 113 KB each hide each other's serial steps, but hold half the cells a pass
+// and double the samples in flight, which then miss L2: 500M-point filtered
+// build 9.6 against 8.3 ms per SM.)
+constexpr int kVoxThreads = 1024;
+constexpr int kVoxWarps = kVoxThreads / 32;
+constexpr int kVoxCtasPerSm = 1;
+constexpr uint32_t kSharedOff = 225 * 1024;       // VoxShared lies behind the arrays
+constexpr int kSmemBytes = 226 * 1024;
+constexpr uint32_t kBatch = 4u * kVoxThreads;  // samples of one CTA iteration
+// 32 KB of occupancy bits (one word per 32 cells along x) and, per word, the
+// 16-bit rank of its first occupied cell
 constexpr uint32_t kWords = kOctCells / 32u;  // 8192
-constexpr uint32_t kDenseOff = kWords * 8u;
-constexpr uint32_t kDenseBytes = kSmemBytes - kDenseOff;
-// cells one accumulate pass holds; every layout ends with the u32 cell of each rank
-constexpr uint32_t kCapSmall = kDenseBytes / 16;   // filtered, <= 65535 points: u64 {R:24 G:24 n:16}, u32 B
-constexpr uint32_t kCapNarrow = kDenseBytes / 20;  // filtered, 32-bit sums: u64 {R, G}, u64 {B, n}
-constexpr uint32_t kCapWide = kDenseBytes / 32;    // filtered, 64-bit sums: 3 x u64, u32 n
-constexpr uint32_t kCapPick = kDenseBytes / 24;    // single sample: {u64 key, u64 payload}, u32 n
+constexpr uint32_t kRankOff = kWords * 4u;
+constexpr uint32_t kDenseOff = kRankOff + kWords * 2u;
+// 16-bit field wraps of one accumulate pass (see update16): a leaf of at most
+// 65,535 points has at most 254 + 255 + 254
+constexpr uint32_t kMaxWraps = 768u;
+constexpr uint32_t kWrapOff = kSharedOff - kMaxWraps * 4u;
+constexpr uint32_t kDenseBytes = kWrapOff - kDenseOff;
+// cells one accumulate pass holds; every layout is 32-bit words (64-bit keys
+// first) followed by the 16-bit cell of each rank.  All updates are native
+// 32-bit shared atomics: a 64-bit shared atomicAdd is a compare-and-swap loop
+// here (measured, 32 lanes on random entries: 18.7 clocks per warp and SM
+// against 2.8 for a 32-bit one, and 125 against 2.6 when the lanes share 32
+// entries; a 64-bit atomicMin is native, 5.2).
+constexpr uint32_t kCapLeaf = kDenseBytes / 10;    // filtered leaf, <= 65535 points: {R:16 G:16}, {B:16 n:16}
+constexpr uint32_t kCapNarrow = kDenseBytes / 18;  // filtered, 32-bit sums: R, G, B, n
+constexpr uint32_t kCapWide = kDenseBytes / 30;    // filtered, 64-bit sums: R, G, B (low and high words), n
+constexpr uint32_t kCapPick = kDenseBytes / 22;    // single sample: u64 {key high word, index}, {index, rgba}, n
 constexpr uint64_t kNarrowMaxSamples = 0xFFFFFFFFull / 255;  // 32-bit channel sums cannot overflow
-constexpr uint64_t kSmallMaxSamples = 0xFFFFu;               // 24-bit sums and a 16-bit count cannot
+constexpr uint64_t kLeafMaxSamples = 0xFFFFu;                // a 16-bit count cannot
 constexpr uint64_t kMask40 = (1ull << 40) - 1;
 constexpr uint32_t kNoRank = 0xFFFFFFFFu;
+constexpr int kScan = (int)(kWords / 4u / kVoxThreads);  // 4-word groups of a thread in the rank scan
 // Filtered staging records of cells of fewer than kPackMaxCount points carry
 // their exact sums in the record's last word (10 bits per channel), so that
 // neither the extraction nor the next level up touches the 16-byte sums
@@ -95,86 +121,31 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// Set the occupancy bits of a thread's four samples (cells with ok[k]).
-// The four bitmap words are read first, back to back, so the thread waits
-// for shared memory once; only bits found clear are then set (most samples
-// find theirs set already).  A read that misses a concurrent update only
-// costs a redundant atomic.
-__device__ __forceinline__ void mark_cells4(uint2* W, const uint32_t (&cell)[4], const bool (&ok)[4]) {
-  uint32_t* w[4];
-  uint32_t bit[4], cur[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    w[k] = &W[cell[k] >> 5].x;  // local cell x | y << 6 | z << 12: word cell / 32
-    bit[k] = 1u << (cell[k] & 31u);
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) cur[k] = ok[k] ? *((volatile uint32_t*)w[k]) : ~0u;
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (!(cur[k] & bit[k])) atomicOr(w[k], bit[k]);
-}
-
 // Ranks, among the item's occupied cells (cell order), of a thread's four
-// samples' cells, minus lo; kNoRank for samples without ok[k] or outside
-// [lo, lo + span).  The bitmap is read-only during an accumulate pass, so
-// the four 8-byte word reads are issued together.
-__device__ __forceinline__ void cell_ranks4(const uint2* W, const uint32_t (&cell)[4], const bool (&ok)[4],
-                                            uint32_t lo, uint32_t span, uint32_t (&rk)[4]) {
-  uint2 e[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) e[k] = ok[k] ? W[cell[k] >> 5] : make_uint2(0u, 0u);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint32_t below = (1u << (cell[k] & 31u)) - 1u;
-    const uint32_t r = e[k].y + __popc(e[k].x & below) - lo;
-    rk[k] = (ok[k] && r < span) ? r : kNoRank;
-  }
-}
-
-// Single-sample modes: the keys of the pick entries of a thread's four
-// ranks, read together before any of them is updated (kNoRank: a key no
-// sample beats).
-template <bool PICKLIKE>
-__device__ __forceinline__ void pre_keys4(const ulonglong2* E, const uint32_t (&rk)[4], uint64_t (&pre)[4]) {
+// samples' cells, minus lo; kNoRank for samples without ok[k] (ALL: every
+// sample counts) or outside [lo, lo + span).  Cells are always valid.  The bitmap is read-only during an accumulate pass, so
+// the reads are issued together.  Word ranks are 16 bits: items of 65,536
+// occupied cells and more (qbase != nullptr) store them relative to the
+// first cell of their quarter of the octant (2048 words).
+template <bool ALL>
+__device__ __forceinline__ void cell_ranks4(const uint32_t* bits, const uint16_t* wrank, const uint32_t* qbase,
+                                            const uint32_t (&cell)[4], const bool* ok, uint32_t lo, uint32_t span,
+                                            uint32_t (&rk)[4]) {
+  uint32_t w[4], b[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    pre[k] = 0ull;
-    if (PICKLIKE && rk[k] != kNoRank) {
-      asm volatile("ld.volatile.shared.u64 %0, [%1];"
-                   : "=l"(pre[k])
-                   : "r"((uint32_t)__cvta_generic_to_shared(E + rk[k])));
-    }
+    w[k] = bits[cell[k] >> 5];
+    b[k] = wrank[cell[k] >> 5];
   }
-}
-
-// Keep the sample of smaller key in a pick entry {key, rgba | index << 32}
-// (keys of distinct samples differ).  `seen` is the entry's key as read
-// earlier: keys only decrease while a pass runs, so a sample whose key is
-// not below that read loses for sure and writes nothing.  Otherwise the
-// entry is read again and the improvement installed with a 128-bit
-// compare-and-swap, retried while others lower the entry meanwhile (each
-// retry sees a strictly smaller key, so the loop ends; the bound only
-// guards against a broken invariant).
-__device__ __forceinline__ bool pick_update(ulonglong2* e, uint64_t h, uint64_t pay, uint64_t seen) {
-  if (h >= seen) return true;
-  const uint32_t addr = (uint32_t)__cvta_generic_to_shared(e);
-  uint64_t c0, c1;
-  asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(c0), "=l"(c1) : "r"(addr) : "memory");
-  for (uint32_t tries = 0; h < c0; ++tries) {
-    if (tries == (1u << 20)) return false;
-    uint64_t p0, p1;
-    asm volatile(
-        "{\n .reg .b128 d, c, s;\n mov.b128 c, {%2, %3};\n mov.b128 s, {%4, %5};\n"
-        " atom.shared.cas.b128 d, [%6], c, s;\n mov.b128 {%0, %1}, d;\n}"
-        : "=l"(p0), "=l"(p1)
-        : "l"(c0), "l"(c1), "l"(h), "l"(pay), "r"(addr)
-        : "memory");
-    if (p0 == c0 && p1 == c1) return true;
-    c0 = p0;
-    c1 = p1;
+  if (qbase) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b[k] += qbase[cell[k] >> 16];
   }
-  return true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t r = b[k] + __popc(w[k] & ((1u << (cell[k] & 31u)) - 1u)) - lo;
+    rk[k] = (ALL || ok[k]) && r < span ? r : kNoRank;
+  }
 }
 
 struct ItemInfo {
@@ -198,13 +169,20 @@ __device__ __forceinline__ uint32_t find_tile(const uint32_t* prefix, uint32_t n
   return lo;
 }
 
-// Local cell (x | y << 6 | z << 12) of a point in the item's octant.
-__device__ __forceinline__ uint32_t point_cell(const int4& q, const ItemInfo& I) {
-  const uint32_t qx = grid_coord((uint32_t)q.x - (uint32_t)I.pmin[0], I.Lp) & 63u;
-  const uint32_t qy = grid_coord((uint32_t)q.y - (uint32_t)I.pmin[1], I.Lp) & 63u;
-  const uint32_t qz = grid_coord((uint32_t)q.z - (uint32_t)I.pmin[2], I.Lp) & 63u;
-  return qx | (qy << 6) | (qz << 12);
-}
+// Local cell (x | y << 6 | z << 12) of a point in the item's octant: bits
+// L - 7 .. L - 2 of each offset from the parent's corner (edge 2^L), moved to
+// their place by one rotation per axis.  Bits that a rotation wraps around
+// are masked off, or zero (L < 7: the offset has no more than L bits).
+struct CellMap {
+  uint32_t mx, my, mz, s;
+  __device__ __forceinline__ explicit CellMap(const ItemInfo& I)
+      : mx((uint32_t)I.pmin[0]), my((uint32_t)I.pmin[1]), mz((uint32_t)I.pmin[2]), s(I.Lp - 7u) {}
+  __device__ __forceinline__ uint32_t operator()(const int4& q) const {
+    const uint32_t dx = (uint32_t)q.x - mx, dy = (uint32_t)q.y - my, dz = (uint32_t)q.z - mz;
+    return (__funnelshift_r(dx, dx, s) & 63u) | (__funnelshift_r(dy, dy, s - 6u) & 0xFC0u) |
+           (__funnelshift_r(dz, dz, s - 12u) & 0x3F000u);
+  }
+};
 
 // Local cell of a child's voxel (its cell in the child's 128^3 grid).
 __device__ __forceinline__ uint32_t voxel_cell(uint32_t cell) {
@@ -234,7 +212,7 @@ int vox_smem_bytes() { return kSmemBytes; }
 
 // Cells per accumulate pass of the four entry layouts (statistics and tests).
 void vox_capacities(uint32_t* small, uint32_t* narrow, uint32_t* wide, uint32_t* pick) {
-  *small = kCapSmall;
+  *small = kCapLeaf;
   *narrow = kCapNarrow;
   *wide = kCapWide;
   *pick = kCapPick;
@@ -244,18 +222,23 @@ void vox_capacities(uint32_t* small, uint32_t* narrow, uint32_t* wide, uint32_t*
 struct VoxShared {
   uint32_t D;                  // occupied cells of the item
   uint32_t r0, r1;             // rank interval this CTA accumulates
-  uint32_t samples;            // samples read by the item's passes (statistics)
-  unsigned long long stage;    // first staging record of the item (rank 0)
   uint32_t nch;                // inner items: children
+  unsigned long long stage;    // first staging record of the item (rank 0)
   int32_t cmin[3];             // header: the child's min corner
+  uint32_t n_wraps;            // 16-bit field wraps listed by the pass
   unsigned long long cparent, cfirst;  // header: parent node, first child (absolute)
   unsigned long long pbase;    // header: the child's first leaf point (absolute)
   uint32_t cpre[9];            // inner items: prefix of the children's record counts
+  uint32_t settle;             // single sample: the pass needs settle_pick
   unsigned long long cstage[8];  // ... their first staging records
   unsigned long long cdense[8];  // ... their places in the voxel array
-  uint32_t wsum[32];
+  uint32_t wsum[kVoxWarps];
+  uint32_t qbase[4];           // rank of the first cell of each quarter of the octant
+  uint32_t pick_level, idx_bound;  // header: level of the parent, bound of the tile's input indices
+  uint32_t next;               // the item or unit taken next
   ItemInfo I;
 };
+static_assert(sizeof(VoxShared) <= kSmemBytes - kSharedOff, "VoxShared fits behind the arrays");
 
 // Reserve `n` consecutive slots of the unit queue; false when it is full
 // (the reservation is all or nothing, so no slot is left unwritten).
@@ -273,24 +256,581 @@ __device__ __forceinline__ bool reserve_units(unsigned int* count, uint32_t cap,
   return false;
 }
 
+// Everything a voxel CTA keeps in shared memory is one dynamic array, so that
+// the phases below (separate functions: each gets the registers for itself)
+// address it as shared memory.
+extern __shared__ __align__(16) unsigned char vox_smem[];
+
+namespace {
+
+__device__ __forceinline__ uint32_t* vox_bits() { return reinterpret_cast<uint32_t*>(vox_smem); }
+__device__ __forceinline__ uint16_t* vox_wrank() { return reinterpret_cast<uint16_t*>(vox_smem + kRankOff); }
+__device__ __forceinline__ uint32_t* vox_fields() { return reinterpret_cast<uint32_t*>(vox_smem + kDenseOff); }
+__device__ __forceinline__ uint32_t* vox_wraps() { return reinterpret_cast<uint32_t*>(vox_smem + kWrapOff); }
+__device__ __forceinline__ VoxShared& vox_shared() { return *reinterpret_cast<VoxShared*>(vox_smem + kSharedOff); }
+
+// The dense entries: one array of `cap` words per field (64-bit keys first),
+// then the 16-bit cell of each rank.
+template <uint32_t WORDS, uint32_t CAP>
+__device__ __forceinline__ uint16_t* vox_cells() {
+  return reinterpret_cast<uint16_t*>(vox_fields() + WORDS * CAP);
+}
+
 // Empty dense entries: all zero bytes in filtered mode (whatever the
-// layout), {~0, 0} and a zero count in the single-sample modes.
+// layout), ~0 keys and zero counts in the single-sample modes.
 template <int MODE>
-__device__ __forceinline__ void vox_clear_dense(unsigned char* smem) {
+__device__ __forceinline__ void vox_clear_dense() {
   if (MODE == LOD_FILTER) {
-    uint4* z = reinterpret_cast<uint4*>(smem + kDenseOff);
-    for (uint32_t i = threadIdx.x; i < kDenseBytes / 16u; i += blockDim.x) z[i] = make_uint4(0, 0, 0, 0);
+    uint4* z = reinterpret_cast<uint4*>(vox_smem + kDenseOff);
+    for (uint32_t i = threadIdx.x; i < kDenseBytes / 16u; i += kVoxThreads) z[i] = make_uint4(0, 0, 0, 0);
   } else {
-    ulonglong2* E = reinterpret_cast<ulonglong2*>(smem + kDenseOff);
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(E + kCapPick);
-    for (uint32_t i = threadIdx.x; i < kCapPick; i += blockDim.x) {
-      E[i] = make_ulonglong2(~0ull, 0ull);
-      cnt[i] = 0u;
+    unsigned long long* E = reinterpret_cast<unsigned long long*>(vox_smem + kDenseOff);
+    for (uint32_t i = threadIdx.x; i < kCapPick; i += kVoxThreads) {
+      E[i] = ~0ull;
+      vox_fields()[4u * kCapPick + i] = 0u;
     }
   }
 }
 
-static_assert(8u * kBlock == kWords, "the rank scan gives every warp 256 words");
+// Set the occupancy bits of a thread's four samples (cells with ok[k]).
+// The four words are read first, back to back, and only bits found clear are
+// set: most samples find theirs set already, and samples that share a word
+// (32 cells in a row, often a whole warp's) then cost one broadcast read
+// where their atomics would be taken one after another.  A read that misses
+// a concurrent update only costs a redundant atomic.
+template <bool ALL>
+__device__ __forceinline__ void mark4(const uint32_t (&cell)[4], const bool* ok) {
+  uint32_t cur[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) cur[k] = ALL || ok[k] ? *((volatile uint32_t*)&vox_bits()[cell[k] >> 5]) : ~0u;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (!((cur[k] >> (cell[k] & 31u)) & 1u)) atomicOr(&vox_bits()[cell[k] >> 5], 1u << (cell[k] & 31u));
+}
+
+__device__ __forceinline__ int4 ld_if(const int4* p, uint32_t tid, int k, uint32_t rem) {
+  int4 q = make_int4(0, 0, 0, 0);
+  if (tid + k * kVoxThreads < rem) q = __ldcg(p + k * kVoxThreads);
+  return q;
+}
+
+// A thread's samples of a contiguous array are p[tid + k * kVoxThreads] for
+// k = 0..3, then the next kBatch: its next four are loaded before its current
+// four are worked on (the item's samples were asked into L2 when it started,
+// so a load is an L2 latency that the other work covers).  `rem` counts the
+// samples from p on, so offsets stay small whatever the item's size.  While
+// two whole batches are left (FULL) no bound is checked.
+
+// Pass 1 (mark the occupied cells) of a leaf's points.
+__device__ __forceinline__ void mark_leaf(const int4* p, uint32_t rem) {
+  const CellMap cm(vox_shared().I);
+  const uint32_t tid = threadIdx.x;
+  p += tid;
+  int4 q0 = ld_if(p, tid, 0, rem), q1 = ld_if(p, tid, 1, rem), q2 = ld_if(p, tid, 2, rem), q3 = ld_if(p, tid, 3, rem);
+  while (rem >= 2 * kBatch) {
+    const uint32_t cell[4] = {cm(q0), cm(q1), cm(q2), cm(q3)};
+    p += kBatch;
+    rem -= kBatch;
+    q0 = __ldcg(p), q1 = __ldcg(p + kVoxThreads), q2 = __ldcg(p + 2 * kVoxThreads), q3 = __ldcg(p + 3 * kVoxThreads);
+    mark4<true>(cell, nullptr);
+  }
+  for (;;) {
+    const uint32_t cell[4] = {cm(q0), cm(q1), cm(q2), cm(q3)};
+    const bool ok[4] = {tid < rem, tid + kVoxThreads < rem, tid + 2 * kVoxThreads < rem, tid + 3 * kVoxThreads < rem};
+    const bool more = rem > kBatch;
+    if (more) {
+      p += kBatch;
+      rem -= kBatch;
+      q0 = ld_if(p, tid, 0, rem), q1 = ld_if(p, tid, 1, rem), q2 = ld_if(p, tid, 2, rem), q3 = ld_if(p, tid, 3, rem);
+    }
+    mark4<false>(cell, ok);
+    if (!more) break;
+  }
+}
+
+// The same with kept indices: the leaf is read from the 32-byte staging
+// records and, when out is given, published to the point / index arrays,
+// contiguously (idempotent: a retried build writes the same values).
+__device__ __forceinline__ void mark_wide(const int4* w, uint32_t rem, int4* out, uint32_t* out_idx) {
+  const CellMap cm(vox_shared().I);
+  const uint32_t tid = threadIdx.x;
+  const bool publish = out != nullptr;
+  w += 2u * tid;
+  out += tid;
+  out_idx += tid;
+  auto load = [&](uint32_t off, int4& q, uint32_t& x) {
+    q = make_int4(0, 0, 0, 0);
+    x = 0u;
+    if (tid + off < rem) ld_wide(w + 2u * off, q, x);
+  };
+  int4 q0, q1, q2, q3;
+  uint32_t x0, x1, x2, x3;
+  load(0, q0, x0), load(kVoxThreads, q1, x1), load(2 * kVoxThreads, q2, x2), load(3 * kVoxThreads, q3, x3);
+  for (;;) {
+    uint32_t cell[4];
+    bool ok[4];
+    auto take = [&](int k, int4& q, uint32_t& x) {
+      ok[k] = tid + k * kVoxThreads < rem;
+      cell[k] = cm(q);
+      if (ok[k] && publish) {
+        out[k * kVoxThreads] = q;
+        out_idx[k * kVoxThreads] = x;
+      }
+      load(kBatch + k * kVoxThreads, q, x);
+    };
+    take(0, q0, x0), take(1, q1, x1), take(2, q2, x2), take(3, q3, x3);
+    mark4<false>(cell, ok);
+    if (rem <= kBatch) break;
+    rem -= kBatch;
+    w += 2u * kBatch;
+    out += kBatch;
+    out_idx += kBatch;
+  }
+}
+
+// The children's voxels, one flat sequence of `total` staged records: child
+// ci of sample f, walking forward.
+__device__ __forceinline__ uint64_t child_record(const VoxShared& S, uint32_t f, uint32_t& ci) {
+  while (f >= S.cpre[ci + 1]) ++ci;
+  return S.cstage[ci] + (f - S.cpre[ci]);
+}
+
+// Pass 1 of an inner child: mark its voxels and, with `dense`, publish them
+// there (idempotent; an array found too small makes the build rerun with the
+// exact size).  Filtered records are published without their packed sums.
+template <bool FILT>
+__device__ __forceinline__ void mark_inner(const int4* stage_in, uint32_t total, int4* dense, uint64_t dense_cap) {
+  const VoxShared& S = vox_shared();
+  uint32_t cl = 0, cp = 0;  // children of the samples being loaded and marked
+  auto load = [&](uint32_t f, int4& q) {
+    q = make_int4(0, 0, 0, 0);
+    if (f < total) q = __ldcg(stage_in + child_record(S, f, cl));
+  };
+  uint32_t f = threadIdx.x;
+  int4 q0, q1, q2, q3;
+  load(f, q0), load(f + kVoxThreads, q1), load(f + 2 * kVoxThreads, q2), load(f + 3 * kVoxThreads, q3);
+  for (; f < total; f += kBatch) {
+    uint32_t cell[4];
+    bool ok[4];
+    auto take = [&](int k, int4& q) {
+      const uint32_t fk = f + k * kVoxThreads;
+      ok[k] = fk < total;
+      cell[k] = voxel_cell((uint32_t)q.x);
+      if (ok[k] && dense) {
+        while (fk >= S.cpre[cp + 1]) ++cp;
+        const uint64_t dst = S.cdense[cp] + (fk - S.cpre[cp]);
+        if (dst < dense_cap) dense[dst] = FILT ? make_int4(q.x, q.y, q.z, (int)kNone) : q;
+      }
+      load(fk + kBatch, q);
+    };
+    take(0, q0), take(1, q1), take(2, q2), take(3, q3);
+    mark4<false>(cell, ok);
+  }
+}
+
+// Pass 2 of a filtered leaf of at most kLeafMaxSamples points: {R:16 G:16}
+// and {B:16 n:16}, two atomics per point.  A 16-bit field that wraps is seen
+// by exactly one of them (in the value it gets back); those wraps, at most
+// kMaxWraps per pass, are listed and put back at extraction.
+template <bool ALL>
+__device__ __forceinline__ void add16x4(const uint32_t (&cell)[4], const uint32_t (&col)[4], const bool* ok, const uint32_t* qbase,
+                                        uint32_t lo, uint32_t span) {
+  VoxShared& S = vox_shared();
+  uint32_t* const W0 = vox_fields();
+  uint32_t* const W1 = W0 + kCapLeaf;
+  uint32_t rk[4], o0[4], o1[4];
+  cell_ranks4<ALL>(vox_bits(), vox_wrank(), qbase, cell, ok, lo, span, rk);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    o0[k] = 0u;
+    o1[k] = 1u;
+    if (rk[k] < span) {
+      o0[k] = atomicAdd(&W0[rk[k]], __byte_perm(col[k], 0u, 0x4140));  // R | G << 16
+      o1[k] = atomicAdd(&W1[rk[k]], __byte_perm(col[k], 1u, 0x5452));  // B | 1 << 16
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (o1[k] == 0u) vox_cells<2, kCapLeaf>()[rk[k]] = (uint16_t)cell[k];
+    if (((o0[k] | o1[k]) & 0x80008000u) == 0u) continue;  // every field below 2^15: nothing wraps
+    const uint32_t r = col[k] & 255u, g = (col[k] >> 8) & 255u, b = (col[k] >> 16) & 255u;
+    const uint32_t wr = ((o0[k] & 0xFFFFu) + r) >> 16, wb = ((o1[k] & 0xFFFFu) + b) >> 16;
+    const uint32_t wg = o0[k] + (r | (g << 16)) < o0[k] ? 1u : 0u;
+    if (wr | wg | wb) {
+      const uint32_t e = atomicAdd(&S.n_wraps, 1u);
+      if (e < kMaxWraps) vox_wraps()[e] = rk[k] | (wr << 16) | (wg << 17) | (wb << 18);
+    }
+  }
+}
+
+__device__ __forceinline__ void acc_leaf16(const int4* p, uint32_t rem, uint32_t lo, uint32_t span) {
+  const CellMap cm(vox_shared().I);
+  const uint32_t* const qbase = vox_shared().D > 0xFFFFu ? vox_shared().qbase : nullptr;
+  const uint32_t tid = threadIdx.x;
+  p += tid;
+  int4 q0 = ld_if(p, tid, 0, rem), q1 = ld_if(p, tid, 1, rem), q2 = ld_if(p, tid, 2, rem), q3 = ld_if(p, tid, 3, rem);
+  while (rem >= 2 * kBatch) {
+    const uint32_t cell[4] = {cm(q0), cm(q1), cm(q2), cm(q3)};
+    const uint32_t col[4] = {(uint32_t)q0.w, (uint32_t)q1.w, (uint32_t)q2.w, (uint32_t)q3.w};
+    p += kBatch;
+    rem -= kBatch;
+    q0 = __ldcg(p), q1 = __ldcg(p + kVoxThreads), q2 = __ldcg(p + 2 * kVoxThreads), q3 = __ldcg(p + 3 * kVoxThreads);
+    add16x4<true>(cell, col, nullptr, qbase, lo, span);
+  }
+  for (;;) {
+    const uint32_t cell[4] = {cm(q0), cm(q1), cm(q2), cm(q3)};
+    const uint32_t col[4] = {(uint32_t)q0.w, (uint32_t)q1.w, (uint32_t)q2.w, (uint32_t)q3.w};
+    const bool ok[4] = {tid < rem, tid + kVoxThreads < rem, tid + 2 * kVoxThreads < rem, tid + 3 * kVoxThreads < rem};
+    const bool more = rem > kBatch;
+    if (more) {
+      p += kBatch;
+      rem -= kBatch;
+      q0 = ld_if(p, tid, 0, rem), q1 = ld_if(p, tid, 1, rem), q2 = ld_if(p, tid, 2, rem), q3 = ld_if(p, tid, 3, rem);
+    }
+    add16x4<false>(cell, col, ok, qbase, lo, span);
+    if (!more) break;
+  }
+}
+
+// One filtered update with full sums: four 32-bit fields (WIDE false), or low
+// and high words (the add that wraps a low word carries) and the count.
+template <bool WIDE>
+__device__ __forceinline__ void add_sums(uint32_t rk, uint32_t cell, uint64_t r, uint64_t g, uint64_t b, uint32_t n) {
+  uint32_t* const F = vox_fields() + rk;
+  if (!WIDE) {
+    atomicAdd(F, (uint32_t)r);
+    atomicAdd(F + kCapNarrow, (uint32_t)g);
+    atomicAdd(F + 2u * kCapNarrow, (uint32_t)b);
+    if (atomicAdd(F + 3u * kCapNarrow, n) == 0u) vox_cells<4, kCapNarrow>()[rk] = (uint16_t)cell;
+  } else {
+    auto add64 = [&](uint32_t f, uint64_t s) {
+      const uint32_t l = (uint32_t)s, old = atomicAdd(F + f * kCapWide, l);
+      const uint32_t h = (uint32_t)(s >> 32) + (old + l < old ? 1u : 0u);
+      if (h) atomicAdd(F + (f + 1u) * kCapWide, h);
+    };
+    add64(0u, r);
+    add64(2u, g);
+    add64(4u, b);
+    if (atomicAdd(F + 6u * kCapWide, n) == 0u) vox_cells<7, kCapWide>()[rk] = (uint16_t)cell;
+  }
+}
+
+// Pass 2 of a filtered leaf of more points.
+template <bool WIDE>
+__device__ __forceinline__ void acc_leaf_sums(const int4* p, uint32_t rem, uint32_t lo, uint32_t span) {
+  VoxShared& S = vox_shared();
+  const CellMap cm(S.I);
+  const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
+  p += threadIdx.x;
+  for (;;) {
+    uint32_t cell[4], rk[4], col[4];
+    bool ok[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      ok[k] = threadIdx.x + k * kVoxThreads < rem;
+      int4 q = make_int4(0, 0, 0, 0);
+      if (ok[k]) q = __ldcg(p + k * kVoxThreads);
+      cell[k] = ok[k] ? cm(q) : 0u;
+      col[k] = (uint32_t)q.w;
+    }
+    cell_ranks4<false>(vox_bits(), vox_wrank(), qbase, cell, ok, lo, span, rk);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (rk[k] != kNoRank) add_sums<WIDE>(rk[k], cell[k], col[k] & 255u, (col[k] >> 8) & 255u, (col[k] >> 16) & 255u, 1u);
+    if (rem <= kBatch) break;
+    rem -= kBatch;
+    p += kBatch;
+  }
+}
+
+// Pass 2 of a filtered inner child: its voxels with their exact sums, which
+// travel in the record (cells of fewer than 1024 points) or lie in the sums
+// array.
+template <bool WIDE>
+__device__ __forceinline__ void acc_inner_sums(const int4* stage_in, const ulonglong2* sums_in, uint32_t total, uint32_t lo,
+                                            uint32_t span) {
+  VoxShared& S = vox_shared();
+  const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
+  uint32_t cl = 0, cs = 0;
+  auto load = [&](uint32_t f, int4& q) {
+    q = make_int4(0, 0, 0, 0);
+    if (f < total) q = __ldcg(stage_in + child_record(S, f, cl));
+  };
+  uint32_t f = threadIdx.x;
+  int4 q0, q1, q2, q3;
+  load(f, q0), load(f + kVoxThreads, q1), load(f + 2 * kVoxThreads, q2), load(f + 3 * kVoxThreads, q3);
+  for (; f < total; f += kBatch) {
+    ulonglong2 sm[4];
+    uint32_t cell[4], rk[4], n[4];
+    bool ok[4];
+    auto take = [&](int k, int4& q) {
+      const uint32_t fk = f + k * kVoxThreads;
+      ok[k] = fk < total;
+      if ((uint32_t)q.w != kNone) sm[k] = unpack_sums(q);
+      else sm[k] = __ldcg(sums_in + child_record(S, fk, cs));
+      cell[k] = voxel_cell((uint32_t)q.x);
+      n[k] = (uint32_t)q.z;
+      load(fk + kBatch, q);
+    };
+    take(0, q0), take(1, q1), take(2, q2), take(3, q3);
+    cell_ranks4<false>(vox_bits(), vox_wrank(), qbase, cell, ok, lo, span, rk);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (rk[k] != kNoRank)
+        add_sums<WIDE>(rk[k], cell[k], sm[k].x & kMask40, (sm[k].x >> 40) | ((sm[k].y & 0xFFFFull) << 24), sm[k].y >> 16, n[k]);
+  }
+}
+
+// Single-sample modes.  Each cell keeps the smallest {high word of the key,
+// input index} (one native 64-bit atomicMin).  A sample that lowered it, and
+// still holds it on a second look, leaves {index, colour} beside it; the
+// extraction takes them when the index is the one kept.  Two things make the
+// pass settle its cells once more by whole keys (settle_pick): two keys of
+// one cell that share their high word (the later update of the two finds the
+// other's word), and a slower sample's {index, colour} written over the
+// winner's.  (Reading the winner back from its position instead of keeping
+// its colour cost more: extraction 1.65 against 0.30 ms per SM on a 200M-point
+// build.)
+struct PickArgs {
+  uint32_t lo, span, level, idx_bound;
+  unsigned long long out_at;  // extraction: staging record of rank lo
+  int4* stage_out;
+  uint64_t stage_cap;
+  unsigned int* error;
+};
+
+__device__ __forceinline__ unsigned long long* pick_keys() { return reinterpret_cast<unsigned long long*>(vox_fields()); }
+__device__ __forceinline__ uint2* pick_pays() { return reinterpret_cast<uint2*>(vox_fields()) + kCapPick; }
+__device__ __forceinline__ uint32_t* pick_counts() { return vox_fields() + 4u * kCapPick; }
+
+template <int MODE>
+__device__ __forceinline__ void pick_sample(const PickArgs& P, uint32_t rk, uint32_t cell, uint32_t ix, uint32_t rgba, uint32_t n) {
+  const uint32_t h = (uint32_t)(pick_key<MODE>(ix, P.level) >> 32);
+  const unsigned long long mine = ((unsigned long long)h << 32) | ix;
+  const unsigned long long old = atomicMin(&pick_keys()[rk], mine);
+  if (atomicAdd(&pick_counts()[rk], n) == 0u) vox_cells<5, kCapPick>()[rk] = (uint16_t)cell;
+  if (old > mine) {
+    if (*((volatile unsigned long long*)&pick_keys()[rk]) == mine) pick_pays()[rk] = make_uint2(ix, rgba);
+  }
+  if ((uint32_t)(old >> 32) == h) vox_shared().settle = 1u;
+}
+
+// A leaf's points and input indices, from the published arrays or (WIDE) the
+// 32-byte staging records.
+template <int MODE, bool WIDE>
+__device__ __forceinline__ void pick_leaf(const PickArgs& P, const int4* p, const uint32_t* pidx, uint32_t total) {
+  VoxShared& S = vox_shared();
+  const CellMap cm(S.I);
+  const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
+  const uint32_t tid = threadIdx.x;
+  uint32_t rem = total;
+  p += (WIDE ? 2u : 1u) * tid;
+  pidx += tid;
+  auto load = [&](uint32_t off, int4& q, uint32_t& x) {
+    q = make_int4(0, 0, 0, 0);
+    x = 0u;
+    if (tid + off < rem) {
+      if (WIDE) {
+        ld_wide_keep(p + 2u * off, q, x);
+      } else {
+        q = __ldcg(p + off);
+        x = __ldcg(pidx + off);
+      }
+    }
+  };
+  int4 q0, q1, q2, q3;
+  uint32_t x0, x1, x2, x3;
+  load(0, q0, x0), load(kVoxThreads, q1, x1), load(2 * kVoxThreads, q2, x2), load(3 * kVoxThreads, q3, x3);
+  for (;;) {
+    uint32_t cell[4], rk[4], ix[4], col[4];
+    bool ok[4];
+    auto take = [&](int k, int4& q, uint32_t& x) {
+      ok[k] = tid + k * kVoxThreads < rem;
+      cell[k] = cm(q);
+      ix[k] = x;
+      col[k] = (uint32_t)q.w;
+      load(kBatch + k * kVoxThreads, q, x);
+    };
+    take(0, q0, x0), take(1, q1, x1), take(2, q2, x2), take(3, q3, x3);
+    cell_ranks4<false>(vox_bits(), vox_wrank(), qbase, cell, ok, P.lo, P.span, rk);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (rk[k] != kNoRank) pick_sample<MODE>(P, rk[k], cell[k], ix[k], col[k], 1u);
+    if (rem <= kBatch) break;
+    rem -= kBatch;
+    p += (WIDE ? 2u : 1u) * kBatch;
+    pidx += kBatch;
+  }
+}
+
+template <int MODE>
+__device__ __forceinline__ void pick_inner(const PickArgs& P, const int4* stage_in, uint32_t total) {
+  VoxShared& S = vox_shared();
+  const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
+  uint32_t cl = 0;
+  auto load = [&](uint32_t f, int4& q) {
+    q = make_int4(0, 0, 0, 0);
+    if (f < total) q = __ldcg(stage_in + child_record(S, f, cl));
+  };
+  uint32_t f = threadIdx.x;
+  int4 q0, q1, q2, q3;
+  load(f, q0), load(f + kVoxThreads, q1), load(f + 2 * kVoxThreads, q2), load(f + 3 * kVoxThreads, q3);
+  for (; f < total; f += kBatch) {
+    uint32_t cell[4], rk[4], ix[4], n[4], col[4];
+    bool ok[4];
+    auto take = [&](int k, int4& q) {
+      const uint32_t fk = f + k * kVoxThreads;
+      ok[k] = fk < total;
+      cell[k] = voxel_cell((uint32_t)q.x);
+      ix[k] = (uint32_t)q.w;
+      n[k] = (uint32_t)q.z;
+      col[k] = (uint32_t)q.y;
+      load(fk + kBatch, q);
+    };
+    take(0, q0), take(1, q1), take(2, q2), take(3, q3);
+    cell_ranks4<false>(vox_bits(), vox_wrank(), qbase, cell, ok, P.lo, P.span, rk);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (rk[k] != kNoRank) pick_sample<MODE>(P, rk[k], cell[k], ix[k], col[k], n[k]);
+  }
+}
+
+// Settles an extracted pass by whole keys: the smallest key of every cell
+// first, then the sample that holds it (keys of distinct samples differ)
+// writes colour and index of the cell's record.  Rare, so it is one sample at
+// a time and keeps its registers to itself.  Every thread of the CTA calls
+// it; the entries are empty before and after.
+template <int MODE>
+__device__ __noinline__ void settle_pick(PickArgs P, const int4* src, const uint32_t* pidx, bool leaf, bool wide, uint32_t total) {
+  VoxShared& S = vox_shared();
+  unsigned long long* const E = pick_keys();
+  const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
+  const CellMap cm(S.I);
+  for (int step = 0; step < 2; ++step) {
+    __syncthreads();
+    uint32_t ci = 0;
+    for (uint32_t i0 = threadIdx.x; i0 < total; i0 += kVoxThreads) {
+      uint32_t cell, rgba, ix;
+      if (leaf) {
+        const int4 q = __ldcg(src + (wide ? 2ull * i0 : (uint64_t)i0));
+        cell = cm(q);
+        rgba = (uint32_t)q.w;
+        ix = __ldcg(wide ? reinterpret_cast<const uint32_t*>(src + 2ull * i0 + 1u) : pidx + i0);
+      } else {
+        const int4 q = __ldcg(src + child_record(S, i0, ci));
+        cell = voxel_cell((uint32_t)q.x);
+        rgba = (uint32_t)q.y;
+        ix = (uint32_t)q.w;
+      }
+      const uint32_t word = cell >> 5;
+      const uint32_t rk = vox_wrank()[word] + (qbase ? qbase[cell >> 16] : 0u) +
+                          __popc(vox_bits()[word] & ((1u << (cell & 31u)) - 1u)) - P.lo;
+      if (rk < P.span) {
+        const unsigned long long key = pick_key<MODE>(ix, P.level);
+        if (step == 0) {
+          atomicMin(&E[rk], key);
+        } else if (E[rk] == key) {
+          if (ix >= P.idx_bound) atomicOr(P.error, kErrInternal);
+          if (P.out_at + rk < P.stage_cap) {
+            P.stage_out[P.out_at + rk].y = (int)rgba;
+            P.stage_out[P.out_at + rk].w = (int)ix;
+          }
+        }
+      }
+      if (total - i0 <= kVoxThreads) break;  // (i0 + kVoxThreads may not fit 32 bits)
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < P.span; i += kVoxThreads) E[i] = ~0ull;
+  if (threadIdx.x == 0) S.settle = 0;
+}
+
+// The cell of rank r (its lower 16 bits are kept beside the entry): the
+// upper two bits are the quarter of the octant the rank lies in.
+__device__ __forceinline__ uint32_t rank_cell(const VoxShared& S, uint32_t low, uint32_t r) {
+  return low | (((r >= S.qbase[1] ? 1u : 0u) + (r >= S.qbase[2] ? 1u : 0u) + (r >= S.qbase[3] ? 1u : 0u)) << 16);
+}
+
+enum SumLayout { kLeaf16, kNarrow, kWide };
+
+// Extraction: rank lo + i goes to staging record at + i (cell order; `at`
+// beyond stage_cap: the reservation reported it), and the entry is left empty
+// for the next pass or item (the next item's layout may put an accumulator
+// where a cell is kept now).
+template <SumLayout LAYOUT>
+__device__ __forceinline__ void extract_sums(int4* stage_out, ulonglong2* sums_out, uint64_t stage_cap, uint64_t at,
+                                          uint32_t lo, uint32_t span) {
+  VoxShared& S = vox_shared();
+  uint32_t* const F = vox_fields();
+  uint16_t* const K = LAYOUT == kLeaf16 ? vox_cells<2, kCapLeaf>() : (LAYOUT == kNarrow ? vox_cells<4, kCapNarrow>() : vox_cells<7, kCapWide>());
+  const uint32_t n_wraps = LAYOUT == kLeaf16 ? min(S.n_wraps, kMaxWraps) : 0u;
+  for (uint32_t i = threadIdx.x; i < span; i += kVoxThreads) {
+    const uint32_t cell = rank_cell(S, K[i], lo + i);
+    K[i] = 0;
+    uint64_t sr, sg, sb, n;
+    if (LAYOUT == kLeaf16) {
+      const uint32_t w0 = F[i], w1 = F[kCapLeaf + i];
+      F[i] = 0u;
+      F[kCapLeaf + i] = 0u;
+      uint32_t cr = 0, cg = 0, cb = 0;
+      for (uint32_t e = 0; e != n_wraps; ++e) {
+        const uint32_t w = vox_wraps()[e];
+        if ((w & 0xFFFFu) == i) {
+          cr += (w >> 16) & 1u;
+          cg += (w >> 17) & 1u;
+          cb += (w >> 18) & 1u;
+        }
+      }
+      // a wrap of a word's lower field has carried into its upper one
+      sr = (w0 & 0xFFFFu) + (cr << 16);
+      sg = (w0 >> 16) + (cg << 16) - cr;
+      sb = (w1 & 0xFFFFu) + (cb << 16);
+      n = ((w1 >> 16) - cb) & 0xFFFFu;
+    } else if (LAYOUT == kNarrow) {
+      sr = F[i];
+      sg = F[kCapNarrow + i];
+      sb = F[2u * kCapNarrow + i];
+      n = F[3u * kCapNarrow + i];
+#pragma unroll
+      for (uint32_t f = 0; f < 4u; ++f) F[f * kCapNarrow + i] = 0u;
+    } else {
+      sr = F[i] | ((uint64_t)F[kCapWide + i] << 32);
+      sg = F[2u * kCapWide + i] | ((uint64_t)F[3u * kCapWide + i] << 32);
+      sb = F[4u * kCapWide + i] | ((uint64_t)F[5u * kCapWide + i] << 32);
+      n = F[6u * kCapWide + i];
+#pragma unroll
+      for (uint32_t f = 0; f < 7u; ++f) F[f * kCapWide + i] = 0u;
+    }
+    const uint32_t m = mean_rgba(sr, sg, sb, n);
+    const bool packed = n < kPackMaxCount;  // the sums travel in the record itself
+    if (at + i < stage_cap) {
+      stage_out[at + i] = make_int4((int)parent_cell(cell, S.I), (int)m, (int)n,
+                                    packed ? (int)pack_remainders(sr, sg, sb, n, m) : (int)kNone);
+      if (!packed) sums_out[at + i] = make_ulonglong2(sr | (sg << 40), (sg >> 24) | (sb << 16));
+    }
+  }
+}
+
+// Extraction of the single-sample modes.
+template <int MODE>
+__device__ __forceinline__ void extract_pick(const PickArgs& P) {
+  VoxShared& S = vox_shared();
+  uint16_t* const K = vox_cells<5, kCapPick>();
+  for (uint32_t i = threadIdx.x; i < P.span; i += kVoxThreads) {
+    const unsigned long long e = pick_keys()[i];
+    const uint2 pay = pick_pays()[i];
+    const uint32_t best = (uint32_t)e, n = pick_counts()[i], cell = rank_cell(S, K[i], P.lo + i);
+    pick_keys()[i] = ~0ull;
+    pick_counts()[i] = 0u;
+    if (pay.x != best) S.settle = 1u;
+    else if (best >= P.idx_bound || (uint32_t)(pick_key<MODE>(best, P.level) >> 32) != (uint32_t)(e >> 32))
+      atomicOr(P.error, kErrInternal);  // cannot happen for a cell that received a sample
+    if (P.out_at + i < P.stage_cap)
+      P.stage_out[P.out_at + i] = make_int4((int)parent_cell(cell, S.I), (int)pay.y, (int)n, (int)best);
+  }
+}
+
+}  // namespace
 
 // Voxelize one item (a child node c of an inner node p at level v.level):
 // all of its ranks, or, for a queued unit (r_unit, p_unit), the ranks
@@ -304,17 +844,17 @@ static_assert(8u * kBlock == kWords, "the rank scan gives every warp 256 words")
 // item split up front, whose leaf may not be published yet (the units of one
 // item run side by side).
 template <int MODE>
-__device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, DevCounters* __restrict__ ctr,
-                                         unsigned char* smem, VoxShared& S, uint32_t it, uint32_t r_unit,
-                                         uint32_t p_unit, bool first, uint32_t* next_item, bool split_unit = false) {
-  uint2* const W = reinterpret_cast<uint2*>(smem);    // {word, rank} per 32 cells
-  uint4* const W4 = reinterpret_cast<uint4*>(smem);   // two of them
+__device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, DevCounters* __restrict__ ctr, uint32_t it,
+                                         uint32_t r_unit, uint32_t p_unit, bool first, uint32_t* next_item,
+                                         bool split_unit = false) {
+  VoxShared& S = vox_shared();
+  uint4* const bits4 = reinterpret_cast<uint4*>(vox_smem);
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   // The item's header, read by warp 0 in two dependent steps: lane 0 reads
   // the child node; then lane 8 reads the parent node while lanes 0..7 read
   // the children's records (inner items), all at once.
-  if (threadIdx.x < 32) {
-    const uint32_t ln = threadIdx.x;
-    if (ln == 0) {
+  if (tid < 32) {
+    if (lane == 0) {
       const uint32_t t = find_tile(v.item_prefix, a.n_tiles, it);
       const uint32_t* ls = v.lvl_start + (uint64_t)t * (kMaxLevels + 1);
       const TileDesc& td = a.tiles[t];
@@ -332,7 +872,8 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       S.cfirst = td.node_base + c.first_child;
       S.pbase = td.pt_base + c.point_offset;
       S.nch = S.I.leaf ? 0u : (uint32_t)__popc(c.child_mask);
-      S.samples = 0;
+      S.pick_level = td.level0 + v.level;
+      S.idx_bound = td.idx_bound;
     }
     __syncwarp();
     const uint32_t nch = S.nch;
@@ -342,10 +883,10 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       const bool wsrc = a.wide != nullptr;
       const char* base = wsrc ? (const char*)(a.wide + 2 * S.pbase) : (const char*)(a.out + S.pbase);
       const uint64_t bytes = umin64(S.I.n * (wsrc ? 32u : 16u), kPrefetchBytes);
-      const uint64_t off = (uint64_t)ln << 16;
+      const uint64_t off = (uint64_t)lane << 16;
       if (off < bytes) prefetch_l2(base + off, (uint32_t)umin64(bytes - off, 1u << 16));
     }
-    if (ln == 8) {
+    if (lane == 8) {
       const lod_node_t p = v.nodes[S.cparent];
       S.I.Lp = p.log2_size;
       S.I.pmin[0] = p.min[0];
@@ -357,162 +898,53 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
     }
     // the children's staged records, one flat sample sequence
     uint32_t occ = 0;
-    if (ln < nch) {
-      const NodeAux ca = v.aux[S.cfirst + ln];
-      S.cstage[ln] = ca.stage;
-      S.cdense[ln] = ca.dense;
+    if (lane < nch) {
+      const NodeAux ca = v.aux[S.cfirst + lane];
+      S.cstage[lane] = ca.stage;
+      S.cdense[lane] = ca.dense;
       occ = ca.occ;
       if (occ) prefetch_l2(v.stage_in + ca.stage, (uint32_t)umin64((uint64_t)occ * 16u, 1u << 16));
     }
-    if (ln < 8) {
+    if (lane < 8) {
       uint32_t incl = occ;  // prefix over lanes 0..7
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xFFu, incl, o);
-        if ((int)ln >= o) incl += y;
+        if ((int)lane >= o) incl += y;
       }
-      if (ln == 0) S.cpre[0] = 0;
-      S.cpre[ln + 1] = incl;
+      if (lane == 0) S.cpre[0] = 0;
+      S.cpre[lane + 1] = incl;
     }
   }
-  for (uint32_t i = threadIdx.x; i < kWords / 2u; i += blockDim.x) W4[i] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (uint32_t i = 0; i < kWords / 4u / kVoxThreads; ++i) bits4[tid + i * kVoxThreads] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  const ItemInfo& I = S.I;
-  const TileDesc& td = a.tiles[I.tile];
-  const lod_node_t& c = v.nodes[I.g];
   constexpr bool PICKLIKE = MODE != LOD_FILTER;  // one sample kept per cell
-  // the narrowest sums that provably cannot overflow for the points of this cube
-  const bool small = MODE == LOD_FILTER && I.npts <= kSmallMaxSamples;
-  const bool narrow = MODE == LOD_FILTER && !small && I.npts <= kNarrowMaxSamples;
-  const bool wide = MODE == LOD_FILTER && !small && !narrow;
-  const uint32_t cap = PICKLIKE ? kCapPick : (small ? kCapSmall : (narrow ? kCapNarrow : kCapWide));
-  const uint32_t C = (v.range_cells && v.range_cells < cap) ? v.range_cells : cap;  // ranks per pass
-  // dense entries, one array per field (64-bit arrays first), then the cell of each rank
-  unsigned char* const dn = smem + kDenseOff;
-  unsigned long long* const A0 = reinterpret_cast<unsigned long long*>(dn);
-  ulonglong2* const E = reinterpret_cast<ulonglong2*>(dn);
-  unsigned long long* A1 = nullptr;
-  unsigned long long* A2 = nullptr;
-  uint32_t* B32 = nullptr;
-  uint32_t* cnt = nullptr;
-  uint32_t* K;
-  if (PICKLIKE) {
-    cnt = reinterpret_cast<uint32_t*>(E + kCapPick);
-    K = cnt + kCapPick;
-  } else if (small) {
-    B32 = reinterpret_cast<uint32_t*>(A0 + kCapSmall);
-    K = B32 + kCapSmall;
-  } else if (narrow) {
-    A1 = A0 + kCapNarrow;
-    K = reinterpret_cast<uint32_t*>(A1 + kCapNarrow);
-  } else {
-    A1 = A0 + kCapWide;
-    A2 = A1 + kCapWide;
-    cnt = reinterpret_cast<uint32_t*>(A2 + kCapWide);
-    K = cnt + kCapWide;
-  }
-
-  const uint64_t pbase = td.pt_base + c.point_offset;
-  const int4* pts = a.out + pbase;
-  const uint32_t* pidx = PICKLIKE ? a.out_idx + pbase : nullptr;
-  // with kept indices the leaf is read from the 32-byte staging records and
-  // published to the point / index arrays here, contiguously
-  const int4* wsrc = a.wide ? a.wide + 2 * pbase : nullptr;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t level = td.level0 + v.level;
+  const bool leaf = S.I.leaf;
   const bool lead = r_unit == 0;  // the one CTA of the item that publishes
-  uint32_t seen = 0;              // samples this thread read (statistics)
-  uint32_t passes = 1;
+  const uint32_t total = leaf ? (uint32_t)S.I.n : S.cpre[S.nch];  // samples
   // the next item's counter value; its latency hides behind the mark pass
   uint32_t next_k = 0;
-  if (next_item && threadIdx.x == 0) next_k = atomicAdd(&ctr->item_head, 1u);
+  if (next_item && tid == 0) next_k = atomicAdd(&ctr->item_head, 1u);
 
   // ---- pass 1: mark the occupied cells
-  if (I.leaf) {
-    const uint64_t n = I.n;
-    const bool publish = wsrc != nullptr && lead;  // idempotent: a retried build writes the same values
-    for (uint64_t base = 0; base < n; base += 4ull * blockDim.x) {
-      int4 q[4];
-      uint32_t x[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint64_t i = base + threadIdx.x + (uint64_t)k * blockDim.x;
-        x[k] = 0u;
-        q[k] = make_int4(0, 0, 0, 0);
-        if (i < n) {
-          if (wsrc) ld_wide_keep(wsrc + 2 * i, q[k], x[k]);
-          else q[k] = __ldcg(pts + i);
-        }
-      }
-      uint32_t cell[4];
-      bool ok[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint64_t i = base + threadIdx.x + (uint64_t)k * blockDim.x;
-        ok[k] = i < n;
-        cell[k] = point_cell(q[k], I);
-        if (ok[k]) {
-          ++seen;
-          if (publish) {
-            a.out[pbase + i] = q[k];
-            a.out_idx[pbase + i] = x[k];
-          }
-        }
-      }
-      mark_cells4(W, cell, ok);
-    }
-  } else {
-    const uint32_t total = S.cpre[S.nch];
-    uint32_t ci = 0;  // child of this thread's current sample (samples only move forward)
-    for (uint32_t f0 = 0; f0 < total; f0 += 4u * blockDim.x) {
-      int4 vr[4];
-      uint64_t dst[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t f = f0 + threadIdx.x + (uint32_t)k * blockDim.x;
-        vr[k] = make_int4(0, 0, 0, 0);
-        dst[k] = 0;
-        if (f < total) {
-          while (f >= S.cpre[ci + 1]) ++ci;
-          vr[k] = __ldcg(v.stage_in + S.cstage[ci] + (f - S.cpre[ci]));
-          dst[k] = S.cdense[ci] + (f - S.cpre[ci]);
-        }
-      }
-      uint32_t cell[4];
-      bool ok[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t f = f0 + threadIdx.x + (uint32_t)k * blockDim.x;
-        ok[k] = f < total;
-        cell[k] = voxel_cell((uint32_t)vr[k].x);
-        if (ok[k]) {
-          ++seen;
-          // publish the child's voxel (idempotent); an array found too
-          // small makes the build rerun with the exact size
-          // (filtered: without the packed sums, pick_index none)
-          if (lead && dst[k] < v.dense_cap)
-            v.dense[dst[k]] = PICKLIKE ? vr[k] : make_int4(vr[k].x, vr[k].y, vr[k].z, (int)kNone);
-        }
-      }
-      mark_cells4(W, cell, ok);
-    }
-  }
+  if (!leaf) mark_inner<!PICKLIKE>(v.stage_in, total, lead ? v.dense : nullptr, v.dense_cap);
+  else if (a.wide) mark_wide(a.wide + 2 * S.pbase, total, lead ? a.out + S.pbase : nullptr, lead ? a.out_idx + S.pbase : nullptr);
+  else mark_leaf(a.out + S.pbase, total);
   __syncthreads();
 
-  // ---- rank the occupied cells: exclusive scan of the words' counts.  Warp
-  // w ranks words [256 w, 256 w + 256), read as pairs {word, rank, word,
-  // rank} by coalesced 16-byte loads: lane l holds pairs l, l + 32, l + 64
-  // and l + 96 of the warp's 128.
+  // ---- rank the occupied cells: exclusive scan of the words' counts.  Every
+  // warp ranks 32 kScan consecutive groups of four words by coalesced 16-byte
+  // loads: lane l holds groups l, l + 32, ...
   uint32_t next_it = next_k;
-  if (next_item && threadIdx.x == 0 && v.order && next_k < v.n_items) next_it = v.order[next_k];
+  if (next_item && tid == 0 && v.order && next_k < v.n_items) next_it = v.order[next_k];
+  uint32_t D;
   {
-    const uint32_t wbase = warp * 128u;
-    uint4 e[4];
-    uint32_t pre[4], tot = 0;
+    uint32_t pre[kScan], tot = 0;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      e[m] = W4[wbase + lane + 32u * (uint32_t)m];
-      const uint32_t c = __popc(e[m].x) + __popc(e[m].z);
+    for (int m = 0; m < kScan; ++m) {
+      const uint4 e = bits4[warp * (32u * kScan) + lane + 32u * (uint32_t)m];
+      const uint32_t c = __popc(e.x) + __popc(e.y) + __popc(e.z) + __popc(e.w);
       uint32_t incl = c;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -524,36 +956,42 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
     }
     if (lane == 0) S.wsum[warp] = tot;
     __syncthreads();
-    if (warp == 0) {
-      const uint32_t w = S.wsum[lane];
-      uint32_t wi = w;
+    // every warp adds up the warps before it
+    const uint32_t ws = lane < kVoxWarps ? S.wsum[lane] : 0u;
+    uint32_t wi = ws;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-        if ((int)lane >= o) wi += y;
-      }
-      S.wsum[lane] = wi - w;
-      if (lane == 31) S.D = wi;
+    for (int o = 1; o < kVoxWarps; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+      if ((int)lane >= o) wi += y;
     }
-    __syncthreads();
-    const uint32_t base = S.wsum[warp];
+    const uint32_t excl = wi - ws;
+    D = __shfl_sync(0xFFFFFFFFu, wi, kVoxWarps - 1);
+    uint32_t base = __shfl_sync(0xFFFFFFFFu, excl, warp);
+    const uint32_t quarter = __shfl_sync(0xFFFFFFFFu, excl, warp & ~(kVoxWarps / 4u - 1u));
+    if (D > 0xFFFFu) base -= quarter;  // word ranks relative to their quarter
+    if (warp == 0 && lane < kVoxWarps && lane % (kVoxWarps / 4u) == 0) S.qbase[lane / (kVoxWarps / 4u)] = excl;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      e[m].y = base + pre[m];
-      e[m].w = e[m].y + __popc(e[m].x);
-      W4[wbase + lane + 32u * (uint32_t)m] = e[m];
+    for (int m = 0; m < kScan; ++m) {
+      const uint32_t at = warp * (32u * kScan) + lane + 32u * (uint32_t)m;
+      const uint4 e = bits4[at];
+      const uint32_t r0 = base + pre[m], r1 = r0 + __popc(e.x), r2 = r1 + __popc(e.y), r3 = r2 + __popc(e.z);
+      reinterpret_cast<uint2*>(vox_wrank())[at] = make_uint2(r0 | (r1 << 16), r2 | (r3 << 16));
     }
   }
+  // the narrowest sums that provably cannot overflow for the points of this cube
+  const SumLayout lay = leaf && S.I.npts <= kLeafMaxSamples ? kLeaf16 : (S.I.npts <= kNarrowMaxSamples ? kNarrow : kWide);
+  const uint32_t cap = PICKLIKE ? kCapPick : (lay == kLeaf16 ? kCapLeaf : (lay == kNarrow ? kCapNarrow : kCapWide));
+  const uint32_t C = (v.range_cells && v.range_cells < cap) ? v.range_cells : cap;  // ranks per pass
   // thread 0: the item's first staging record.  The reservation (or, for
   // a unit, the read of the first attempt's) is issued here and its value
   // first used before the first extraction, so its latency overlaps the
   // accumulate pass.
   unsigned long long stg = 0;
-  if (threadIdx.x == 0) {
-    const uint32_t D = S.D;
+  if (tid == 0) {
+    S.D = D;
     if (first) {
       stg = atomicAdd(v.stage_used, (unsigned long long)D);
-      v.aux[I.g].occ = D;
+      v.aux[S.I.g].occ = D;
       S.r0 = 0;
       S.r1 = D;
       const uint32_t P = (D + C - 1) / C;
@@ -564,337 +1002,118 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
         S.r1 = D / P;
       }
     } else {
-      stg = v.aux[I.g].stage;  // reserved by the first attempt, or by the up-front split
+      stg = v.aux[S.I.g].stage;  // reserved by the first attempt, or by the up-front split
       S.r0 = (uint32_t)((uint64_t)D * r_unit / p_unit);
       S.r1 = (uint32_t)((uint64_t)D * (r_unit + 1) / p_unit);
-      if (r_unit == 0) v.aux[I.g].occ = D;
+      if (r_unit == 0) v.aux[S.I.g].occ = D;
     }
+    S.n_wraps = 0;
+    S.settle = 0;
   }
   __syncthreads();
-  const uint32_t r1 = S.r1;
-  const bool merge = !PICKLIKE && !wide && !v.no_merge;
-
-  // Filtered, 32-bit sums (merge): runs of consecutive lanes whose k-th
-  // samples share a rank (points in scan order often do) add their sums
-  // first, so that only the run's first lane updates the entry (at most 32
-  // samples of 8-bit channels or the sums of one cell, which the layout
-  // bounds).  The four samples of a thread are reduced side by side
-  // (segmented suffix sums by doubling, only as many steps as the longest
-  // run needs); a warp without runs pays four shuffles and four votes.
-  // dt[k] is cleared for the lanes whose sums went to another lane.
-  auto merge4 = [&](const uint32_t (&rk)[4], uint32_t (&vr)[4], uint32_t (&vg)[4], uint32_t (&vb)[4],
-                    uint32_t (&vn)[4], bool (&dt)[4]) {
-    unsigned dm[4];  // bit i: lane i + 1 continues lane i's run
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint32_t nxt = __shfl_down_sync(0xFFFFFFFFu, rk[k], 1);
-      dm[k] = __ballot_sync(0xFFFFFFFFu, lane < 31u && dt[k] && nxt == rk[k]);
-    }
-    uint32_t x = dm[0] | dm[1] | dm[2] | dm[3];
-    if (!x) return;
-    uint32_t longest = 0;  // longest run of set bits (an upper bound over the four masks)
-    while (x) {
-      x &= x >> 1;
-      ++longest;
-    }
-    uint32_t end[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) end[k] = (uint32_t)__ffs(~dm[k] & (0xFFFFFFFFu << lane)) - 1u;  // last lane of the run
-    for (uint32_t o = 1; o <= longest; o <<= 1) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (!dm[k]) continue;  // warp-uniform
-        const uint32_t tr = __shfl_down_sync(0xFFFFFFFFu, vr[k], o), tg = __shfl_down_sync(0xFFFFFFFFu, vg[k], o);
-        const uint32_t tb = __shfl_down_sync(0xFFFFFFFFu, vb[k], o), tn = __shfl_down_sync(0xFFFFFFFFu, vn[k], o);
-        if (lane + o <= end[k]) {
-          vr[k] += tr;
-          vg[k] += tg;
-          vb[k] += tb;
-          vn[k] += tn;
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) dt[k] = dt[k] && (lane == 0 || !((dm[k] >> (lane - 1)) & 1u));
-  };
-
-  // update the dense entry of rank rk with one sample (or a run's sums).
-  // Single-sample modes: pre is the entry's key as read before (see pick_update).
-  auto update = [&](uint32_t rk, uint32_t cell, uint64_t r, uint64_t g, uint64_t b, uint32_t n, uint32_t ix,
-                    uint32_t rgba, uint64_t pre) {
-    K[rk] = cell;
-    if (PICKLIKE) {
-      if (!pick_update(&E[rk], pick_key<MODE>(ix, level), (uint64_t)rgba | ((uint64_t)ix << 32), pre))
-        atomicOr(&ctr->error, kErrInternal);
-      atomicAdd(&cnt[rk], n);
-    } else if (small) {
-      atomicAdd(&A0[rk], r | (g << 24) | ((uint64_t)n << 48));
-      atomicAdd(&B32[rk], (uint32_t)b);
-    } else if (narrow) {
-      atomicAdd(&A0[rk], r | (g << 32));
-      atomicAdd(&A1[rk], b | ((uint64_t)n << 32));
-    } else {
-      atomicAdd(&A0[rk], r);
-      atomicAdd(&A1[rk], g);
-      atomicAdd(&A2[rk], b);
-      atomicAdd(&cnt[rk], n);
-    }
-  };
 
   // ---- pass 2: accumulate the ranks [lo, lo + span), one pass per range
   // a leaf read from 32-byte staging records is published (points and
   // indices, 20 bytes) by the mark pass of its first attempt: later passes
   // read the published copy
-  const bool from_wide = wsrc != nullptr && split_unit;
-  for (uint32_t lo = S.r0; lo < r1; lo += C) {
+  const bool from_wide = PICKLIKE && split_unit;
+  uint32_t passes = 1;
+  for (uint32_t lo = S.r0, r1 = S.r1; lo < r1; lo += C) {
     const uint32_t span = r1 - lo < C ? r1 - lo : C;
-    const bool last = r1 - lo <= C;  // the item's last read: let it leave L2 first
     ++passes;
-    if (I.leaf) {
-      const uint64_t n = I.n;
-      for (uint64_t base = 0; base < n; base += 4ull * blockDim.x) {
-        int4 q[4];
-        uint32_t x[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint64_t i = base + threadIdx.x + (uint64_t)k * blockDim.x;
-          x[k] = 0u;
-          q[k] = make_int4(0, 0, 0, 0);
-          if (i < n) {
-            if (from_wide) {
-              if (last) ld_wide(wsrc + 2 * i, q[k], x[k]);
-              else ld_wide_keep(wsrc + 2 * i, q[k], x[k]);
-            } else {
-              q[k] = last ? __ldcs(pts + i) : __ldcg(pts + i);
-              if (PICKLIKE) x[k] = last ? __ldcs(pidx + i) : __ldcg(pidx + i);
-            }
-          }
-        }
-        uint32_t cell[4], rk[4];
-        bool ok[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint64_t i = base + threadIdx.x + (uint64_t)k * blockDim.x;
-          ok[k] = i < n;
-          seen += ok[k] ? 1u : 0u;
-          cell[k] = point_cell(q[k], I);
-        }
-        cell_ranks4(W, cell, ok, lo, span, rk);
-        uint64_t pre[4];
-        pre_keys4<PICKLIKE>(E, rk, pre);
-        uint32_t vr[4], vg[4], vb[4], vn[4];
-        bool dt[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint32_t rgba = (uint32_t)q[k].w;
-          vr[k] = rgba & 255u;
-          vg[k] = (rgba >> 8) & 255u;
-          vb[k] = (rgba >> 16) & 255u;
-          vn[k] = 1u;
-          dt[k] = rk[k] != kNoRank;
-        }
-        if (merge) merge4(rk, vr, vg, vb, vn, dt);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (dt[k]) update(rk[k], cell[k], vr[k], vg[k], vb[k], vn[k], x[k], (uint32_t)q[k].w, pre[k]);
-      }
+    const int4* const src = !leaf ? v.stage_in : (from_wide ? a.wide + 2 * S.pbase : a.out + S.pbase);
+    const uint32_t* const pidx = PICKLIKE ? a.out_idx + S.pbase : nullptr;
+    PickArgs P;
+    if (PICKLIKE) {
+      P.lo = lo;
+      P.span = span;
+      P.level = S.pick_level;
+      P.idx_bound = S.idx_bound;
+      P.stage_out = v.stage_out;
+      P.stage_cap = v.stage_cap;
+      P.error = &ctr->error;
+      P.out_at = 0;
+      if (!leaf) pick_inner<MODE>(P, src, total);
+      else if (from_wide) pick_leaf<MODE, true>(P, src, pidx, total);
+      else pick_leaf<MODE, false>(P, src, pidx, total);
+    } else if (leaf) {
+      if (lay == kLeaf16) acc_leaf16(src, total, lo, span);
+      else if (lay == kNarrow) acc_leaf_sums<false>(src, total, lo, span);
+      else acc_leaf_sums<true>(src, total, lo, span);
     } else {
-      const uint32_t total = S.cpre[S.nch];
-      uint32_t ci = 0;
-      for (uint32_t f0 = 0; f0 < total; f0 += 4u * blockDim.x) {
-        int4 vr[4];
-        ulonglong2 sm[4];
-        uint64_t src[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint32_t f = f0 + threadIdx.x + (uint32_t)k * blockDim.x;
-          vr[k] = make_int4(0, 0, 0, 0);
-          sm[k] = make_ulonglong2(0ull, 0ull);
-          src[k] = 0;
-          if (f < total) {
-            while (f >= S.cpre[ci + 1]) ++ci;
-            src[k] = S.cstage[ci] + (f - S.cpre[ci]);
-            vr[k] = last ? __ldcs(v.stage_in + src[k]) : __ldcg(v.stage_in + src[k]);
-          }
-        }
-        if (!PICKLIKE) {
-          // exact sums: in the record (cells of fewer than 1024 points), else
-          // in the sums array
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint32_t f = f0 + threadIdx.x + (uint32_t)k * blockDim.x;
-            if (f >= total) continue;
-            if ((uint32_t)vr[k].w != kNone) sm[k] = unpack_sums(vr[k]);
-            else sm[k] = last ? __ldcs(v.stage_in_sum + src[k]) : __ldcg(v.stage_in_sum + src[k]);
-          }
-        }
-        uint32_t cell[4], rk[4];
-        bool ok[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint32_t f = f0 + threadIdx.x + (uint32_t)k * blockDim.x;
-          ok[k] = f < total;
-          seen += ok[k] ? 1u : 0u;
-          cell[k] = voxel_cell((uint32_t)vr[k].x);
-        }
-        cell_ranks4(W, cell, ok, lo, span, rk);
-        uint64_t pre[4];
-        pre_keys4<PICKLIKE>(E, rk, pre);
-        // a child's voxel: {cell, rgba, count, picked index} and packed exact sums
-        bool dt[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) dt[k] = rk[k] != kNoRank;
-        if (merge) {
-          uint32_t mr[4], mg[4], mb[4], mn[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            mr[k] = (uint32_t)(sm[k].x & kMask40);
-            mg[k] = (uint32_t)((sm[k].x >> 40) | ((sm[k].y & 0xFFFFull) << 24));
-            mb[k] = (uint32_t)(sm[k].y >> 16);
-            mn[k] = (uint32_t)vr[k].z;
-          }
-          merge4(rk, mr, mg, mb, mn, dt);
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (dt[k]) update(rk[k], cell[k], mr[k], mg[k], mb[k], mn[k], 0u, 0u, 0ull);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint64_t sr = sm[k].x & kMask40, sg = (sm[k].x >> 40) | ((sm[k].y & 0xFFFFull) << 24),
-                           sb = sm[k].y >> 16;
-            if (dt[k]) update(rk[k], cell[k], sr, sg, sb, (uint32_t)vr[k].z, (uint32_t)vr[k].w, (uint32_t)vr[k].y, pre[k]);
-          }
-        }
-      }
+      if (lay == kNarrow) acc_inner_sums<false>(src, v.stage_in_sum, total, lo, span);
+      else acc_inner_sums<true>(src, v.stage_in_sum, total, lo, span);
     }
-    if (threadIdx.x == 0) S.stage = stg;
+    if (tid == 0) S.stage = stg;
     __syncthreads();  // every update of the pass is done
-    const unsigned long long stage = S.stage;
-
-    // ---- extract: rank lo + i goes to staging record stage + lo + i (cell
-    // order), and the entry is left empty for the next pass or item
-    for (uint32_t i = threadIdx.x; i < span; i += blockDim.x) {
-      const uint32_t cell = K[i];
-      const uint64_t o = stage + lo + i;
-      int4 rec;
-      rec.x = (int)parent_cell(cell, I);
-      ulonglong2 sums = make_ulonglong2(0ull, 0ull);
-      bool packed = false;  // filtered: the sums travel in the record itself
-      if (PICKLIKE) {
-        const ulonglong2 e = E[i];
-        const uint32_t c32 = cnt[i];
-        E[i] = make_ulonglong2(~0ull, 0ull);
-        cnt[i] = 0u;
-        const uint32_t best = (uint32_t)(e.y >> 32);
-        if (best >= td.idx_bound || pick_key<MODE>(best, level) != e.x) {
-          atomicOr(&ctr->error, kErrInternal);  // cannot happen for a cell that received a sample
-          continue;
-        }
-        rec.y = (int)(uint32_t)e.y;
-        rec.z = (int)c32;
-        rec.w = (int)best;
-      } else {
-        uint64_t sr, sg, sb, n;
-        if (small) {
-          const uint64_t a0 = A0[i];
-          sr = a0 & 0xFFFFFFull;
-          sg = (a0 >> 24) & 0xFFFFFFull;
-          n = a0 >> 48;
-          sb = B32[i];
-          A0[i] = 0ull;
-          B32[i] = 0u;
-        } else if (narrow) {
-          const uint64_t a0 = A0[i], a1 = A1[i];
-          sr = a0 & 0xFFFFFFFFull;
-          sg = a0 >> 32;
-          sb = a1 & 0xFFFFFFFFull;
-          n = a1 >> 32;
-          A0[i] = 0ull;
-          A1[i] = 0ull;
-        } else {
-          sr = A0[i];
-          sg = A1[i];
-          sb = A2[i];
-          n = cnt[i];
-          A0[i] = 0ull;
-          A1[i] = 0ull;
-          A2[i] = 0ull;
-          cnt[i] = 0u;
-        }
-        K[i] = 0u;  // the next item's layout may put an accumulator here
-        const uint32_t m = mean_rgba(sr, sg, sb, n);
-        rec.y = (int)m;
-        rec.z = (int)n;
-        rec.w = (int)kNone;
-        if (n < kPackMaxCount) {
-          rec.w = (int)pack_remainders(sr, sg, sb, n, m);
-          packed = true;
-        } else {
-          sums.x = sr | (sg << 40);
-          sums.y = (sg >> 24) | (sb << 16);
-        }
-      }
-      if (o < v.stage_cap) {  // else the reservation reported kErrStageCap
-        v.stage_out[o] = rec;
-        if (!PICKLIKE && !packed) v.stage_out_sum[o] = sums;
-      }
+    const unsigned long long at = S.stage + lo;
+    if (PICKLIKE) {
+      P.out_at = at;
+      extract_pick<MODE>(P);
+      __syncthreads();
+      if (S.settle) settle_pick<MODE>(P, src, pidx, leaf, from_wide, total);
+    } else if (lay == kLeaf16) {
+      extract_sums<kLeaf16>(v.stage_out, v.stage_out_sum, v.stage_cap, at, lo, span);
+    } else if (lay == kNarrow) {
+      extract_sums<kNarrow>(v.stage_out, v.stage_out_sum, v.stage_cap, at, lo, span);
+    } else {
+      extract_sums<kWide>(v.stage_out, v.stage_out_sum, v.stage_cap, at, lo, span);
     }
     __syncthreads();
+    if (!PICKLIKE && lay == kLeaf16 && r1 - lo > C) {  // more passes follow: they list their own wraps
+      if (tid == 0) S.n_wraps = 0;
+      __syncthreads();
+    }
   }
-  seen = __reduce_add_sync(0xFFFFFFFFu, seen);
-  if (lane == 0 && seen) atomicAdd(&S.samples, seen);
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     if (first) {
-      v.aux[I.g].stage = stg;
-      if (stg + S.D > v.stage_cap) atomicOr(&ctr->error, kErrStageCap);
+      v.aux[S.I.g].stage = stg;
+      if (stg + D > v.stage_cap) atomicOr(&ctr->error, kErrStageCap);
     }
     if (next_item) *next_item = next_it;  // read after this item's last barrier
     atomicAdd(&ctr->vox_passes, (unsigned long long)passes);
-    atomicAdd(&ctr->vox_samples, (unsigned long long)S.samples);
-    if (first) atomicMax(&ctr->vox_max_item, (unsigned long long)I.n);
+    atomicAdd(&ctr->vox_samples, (unsigned long long)passes * total);
+    if (first) atomicMax(&ctr->vox_max_item, (unsigned long long)S.I.n);
   }
   __syncthreads();
 }
 
-// First attempt of every item, taken by persistent CTAs (one per SM: the
-// bitmap and the dense entries fill the shared memory) in the level's item
+// First attempt of every item, taken by persistent CTAs in the level's item
 // order.  While an item is marked, its CTA already takes the next one.
 template <int MODE>
-__global__ void __launch_bounds__(kBlock, 1) k_vox(BuildArgs a, VoxLevel v, DevCounters* __restrict__ ctr) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ VoxShared S;
-  __shared__ uint32_t s_item;
-  vox_clear_dense<MODE>(smem);
+__global__ void __launch_bounds__(kVoxThreads, kVoxCtasPerSm)
+    k_vox(const __grid_constant__ BuildArgs a, const __grid_constant__ VoxLevel v, DevCounters* __restrict__ ctr) {
+  VoxShared& S = vox_shared();
+  vox_clear_dense<MODE>();
   if (threadIdx.x == 0) {
     const uint32_t k = atomicAdd(&ctr->item_head, 1u);
-    s_item = (v.order && k < v.n_items) ? v.order[k] : k;
+    S.next = (v.order && k < v.n_items) ? v.order[k] : k;
   }
   __syncthreads();
   for (;;) {
-    const uint32_t it = s_item;  // every thread reads it before the item's first barrier
+    const uint32_t it = S.next;  // every thread reads it before the item's first barrier
     if (it >= v.n_items) break;
-    vox_item<MODE>(a, v, ctr, smem, S, it, 0u, 1u, true, &s_item);
+    vox_item<MODE>(a, v, ctr, it, 0u, 1u, true, &S.next);
   }
 }
 
 // Rank ranges of items with many occupied cells, taken from the queue by
 // persistent CTAs (the queue is complete when this starts).
 template <int MODE>
-__global__ void __launch_bounds__(kBlock, 1) k_vox_units(BuildArgs a, VoxLevel v, DevCounters* __restrict__ ctr) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ VoxShared S;
-  __shared__ uint32_t s_unit;
+__global__ void __launch_bounds__(kVoxThreads, kVoxCtasPerSm)
+    k_vox_units(const __grid_constant__ BuildArgs a, const __grid_constant__ VoxLevel v, DevCounters* __restrict__ ctr) {
+  VoxShared& S = vox_shared();
   const uint32_t n_units = min(ctr->units, v.unit_cap);
-  vox_clear_dense<MODE>(smem);
+  if (blockIdx.x >= n_units) return;
+  vox_clear_dense<MODE>();
   for (;;) {
-    if (threadIdx.x == 0) s_unit = atomicAdd(&ctr->unit_head, 1u);
+    if (threadIdx.x == 0) S.next = atomicAdd(&ctr->unit_head, 1u);
     __syncthreads();
-    const uint32_t u = s_unit;
+    const uint32_t u = S.next;
     __syncthreads();
     if (u >= n_units) break;
     const uint4 w = v.units[u];
-    vox_item<MODE>(a, v, ctr, smem, S, w.x, w.y, w.z, false, nullptr, w.w != 0u);
+    vox_item<MODE>(a, v, ctr, w.x, w.y, w.z, false, nullptr, w.w != 0u);
   }
 }
 
@@ -947,19 +1166,19 @@ int vox_init() {
 
 template <int MODE>
 static cudaError_t launch_vox_mode(const BuildArgs& a, const VoxLevel& v, DevCounters* ctr, cudaStream_t st) {
-  const int sms = vox_init();
-  if (v.units && v.n_items * 4u <= (uint32_t)sms) {
+  const uint32_t ctas = (uint32_t)(vox_init() * kVoxCtasPerSm);
+  if (v.units && v.n_items * 4u <= ctas) {
     uint32_t m = 0;
-    while (m < 3 && (v.n_items << (m + 1)) <= (uint32_t)sms) ++m;
+    while (m < 3 && (v.n_items << (m + 1)) <= ctas) ++m;
     k_vox_split<<<(v.n_items + 127) / 128, 128, 0, st>>>(a, v, ctr, m);
     note_launch();
-    k_vox_units<MODE><<<sms, kBlock, kSmemBytes, st>>>(a, v, ctr);
+    k_vox_units<MODE><<<ctas, kVoxThreads, kSmemBytes, st>>>(a, v, ctr);
     note_launch();
     return cudaGetLastError();
   }
-  k_vox<MODE><<<v.n_items < (uint32_t)sms ? v.n_items : (uint32_t)sms, kBlock, kSmemBytes, st>>>(a, v, ctr);
+  k_vox<MODE><<<v.n_items < ctas ? v.n_items : ctas, kVoxThreads, kSmemBytes, st>>>(a, v, ctr);
   note_launch();
-  if (v.units) k_vox_units<MODE><<<sms, kBlock, kSmemBytes, st>>>(a, v, ctr);
+  if (v.units) k_vox_units<MODE><<<ctas, kVoxThreads, kSmemBytes, st>>>(a, v, ctr);
   if (v.units) note_launch();
   return cudaGetLastError();
 }
