@@ -195,17 +195,6 @@ __device__ __forceinline__ uint32_t parent_cell(uint32_t l, const ItemInfo& I) {
   return ((I.kx << 6) | (l & 63u)) | (((I.ky << 6) | ((l >> 6) & 63u)) << 7) | (((I.kz << 6) | (l >> 12)) << 14);
 }
 
-// One 32-byte {point, index} record, kept in L2 (it is read again).
-__device__ __forceinline__ void ld_wide_keep(const int4* p, int4& q, uint32_t& idx) {
-  uint32_t u0, u1, u2;
-  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w), "=r"(idx), "=r"(u0), "=r"(u1), "=r"(u2)
-      : "l"(p));
-  (void)u0;
-  (void)u1;
-  (void)u2;
-}
-
 }  // namespace
 
 int vox_smem_bytes() { return kSmemBytes; }
@@ -615,27 +604,22 @@ __device__ __forceinline__ void pick_sample(const PickArgs& P, uint32_t rk, uint
   if ((uint32_t)(old >> 32) == h) vox_shared().settle = 1u;
 }
 
-// A leaf's points and input indices, from the published arrays or (WIDE) the
-// 32-byte staging records.
-template <int MODE, bool WIDE>
+// A leaf's points and input indices.
+template <int MODE>
 __device__ __forceinline__ void pick_leaf(const PickArgs& P, const int4* p, const uint32_t* pidx, uint32_t total) {
   VoxShared& S = vox_shared();
   const CellMap cm(S.I);
   const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
   const uint32_t tid = threadIdx.x;
   uint32_t rem = total;
-  p += (WIDE ? 2u : 1u) * tid;
+  p += tid;
   pidx += tid;
   auto load = [&](uint32_t off, int4& q, uint32_t& x) {
     q = make_int4(0, 0, 0, 0);
     x = 0u;
     if (tid + off < rem) {
-      if (WIDE) {
-        ld_wide_keep(p + 2u * off, q, x);
-      } else {
-        q = __ldcg(p + off);
-        x = __ldcg(pidx + off);
-      }
+      q = __ldcg(p + off);
+      x = __ldcg(pidx + off);
     }
   };
   int4 q0, q1, q2, q3;
@@ -658,7 +642,7 @@ __device__ __forceinline__ void pick_leaf(const PickArgs& P, const int4* p, cons
       if (rk[k] != kNoRank) pick_sample<MODE>(P, rk[k], cell[k], ix[k], col[k], 1u);
     if (rem <= kBatch) break;
     rem -= kBatch;
-    p += (WIDE ? 2u : 1u) * kBatch;
+    p += kBatch;
     pidx += kBatch;
   }
 }
@@ -701,7 +685,7 @@ __device__ __forceinline__ void pick_inner(const PickArgs& P, const int4* stage_
 // a time and keeps its registers to itself.  Every thread of the CTA calls
 // it; the entries are empty before and after.
 template <int MODE>
-__device__ __noinline__ void settle_pick(PickArgs P, const int4* src, const uint32_t* pidx, bool leaf, bool wide, uint32_t total) {
+__device__ __noinline__ void settle_pick(PickArgs P, const int4* src, const uint32_t* pidx, bool leaf, uint32_t total) {
   VoxShared& S = vox_shared();
   unsigned long long* const E = pick_keys();
   const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
@@ -712,10 +696,10 @@ __device__ __noinline__ void settle_pick(PickArgs P, const int4* src, const uint
     for (uint32_t i0 = threadIdx.x; i0 < total; i0 += kVoxThreads) {
       uint32_t cell, rgba, ix;
       if (leaf) {
-        const int4 q = __ldcg(src + (wide ? 2ull * i0 : (uint64_t)i0));
+        const int4 q = __ldcg(src + i0);
         cell = cm(q);
         rgba = (uint32_t)q.w;
-        ix = __ldcg(wide ? reinterpret_cast<const uint32_t*>(src + 2ull * i0 + 1u) : pidx + i0);
+        ix = __ldcg(pidx + i0);
       } else {
         const int4 q = __ldcg(src + child_record(S, i0, ci));
         cell = voxel_cell((uint32_t)q.x);
@@ -841,8 +825,7 @@ __device__ __forceinline__ void extract_pick(const PickArgs& P) {
 // publishes what it reads (the leaf's points, the children's voxels).
 // `next_item` (first attempts): where thread 0 leaves the item the CTA
 // takes next, fetched while this one is marked.  `split_unit`: a range of an
-// item split up front, whose leaf may not be published yet (the units of one
-// item run side by side).
+// item split up front.
 template <int MODE>
 __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, DevCounters* __restrict__ ctr, uint32_t it,
                                          uint32_t r_unit, uint32_t p_unit, bool first, uint32_t* next_item,
@@ -921,7 +904,10 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
   __syncthreads();
   constexpr bool PICKLIKE = MODE != LOD_FILTER;  // one sample kept per cell
   const bool leaf = S.I.leaf;
-  const bool lead = r_unit == 0;  // the one CTA of the item that publishes
+  const bool lead = r_unit == 0;  // the one CTA of the item that publishes the children's voxels
+  // the units of an item split up front run side by side, so each of them
+  // publishes the leaf (the same values) that its later passes read
+  const bool own_leaf = lead || split_unit;
   const uint32_t total = leaf ? (uint32_t)S.I.n : S.cpre[S.nch];  // samples
   // the next item's counter value; its latency hides behind the mark pass
   uint32_t next_k = 0;
@@ -929,7 +915,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
 
   // ---- pass 1: mark the occupied cells
   if (!leaf) mark_inner<!PICKLIKE>(v.stage_in, total, lead ? v.dense : nullptr, v.dense_cap);
-  else if (a.wide) mark_wide(a.wide + 2 * S.pbase, total, lead ? a.out + S.pbase : nullptr, lead ? a.out_idx + S.pbase : nullptr);
+  else if (a.wide) mark_wide(a.wide + 2 * S.pbase, total, own_leaf ? a.out + S.pbase : nullptr, own_leaf ? a.out_idx + S.pbase : nullptr);
   else mark_leaf(a.out + S.pbase, total);
   __syncthreads();
 
@@ -1013,15 +999,13 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
   __syncthreads();
 
   // ---- pass 2: accumulate the ranks [lo, lo + span), one pass per range
-  // a leaf read from 32-byte staging records is published (points and
-  // indices, 20 bytes) by the mark pass of its first attempt: later passes
-  // read the published copy
-  const bool from_wide = PICKLIKE && split_unit;
+  // (a leaf read from 32-byte staging records was published by the mark pass:
+  // later passes read the 16- or 20-byte copy)
   uint32_t passes = 1;
   for (uint32_t lo = S.r0, r1 = S.r1; lo < r1; lo += C) {
     const uint32_t span = r1 - lo < C ? r1 - lo : C;
     ++passes;
-    const int4* const src = !leaf ? v.stage_in : (from_wide ? a.wide + 2 * S.pbase : a.out + S.pbase);
+    const int4* const src = leaf ? a.out + S.pbase : v.stage_in;
     const uint32_t* const pidx = PICKLIKE ? a.out_idx + S.pbase : nullptr;
     PickArgs P;
     if (PICKLIKE) {
@@ -1034,8 +1018,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       P.error = &ctr->error;
       P.out_at = 0;
       if (!leaf) pick_inner<MODE>(P, src, total);
-      else if (from_wide) pick_leaf<MODE, true>(P, src, pidx, total);
-      else pick_leaf<MODE, false>(P, src, pidx, total);
+      else pick_leaf<MODE>(P, src, pidx, total);
     } else if (leaf) {
       if (lay == kLeaf16) acc_leaf16(src, total, lo, span);
       else if (lay == kNarrow) acc_leaf_sums<false>(src, total, lo, span);
@@ -1051,7 +1034,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       P.out_at = at;
       extract_pick<MODE>(P);
       __syncthreads();
-      if (S.settle) settle_pick<MODE>(P, src, pidx, leaf, from_wide, total);
+      if (S.settle) settle_pick<MODE>(P, src, pidx, leaf, total);
     } else if (lay == kLeaf16) {
       extract_sums<kLeaf16>(v.stage_out, v.stage_out_sum, v.stage_cap, at, lo, span);
     } else if (lay == kNarrow) {
