@@ -119,6 +119,7 @@ struct DevCounters {
   unsigned long long vox_passes;      // passes over samples (mark and accumulate) of all voxel items
   unsigned long long vox_samples;     // samples read by all table passes (re-reads included)
   unsigned long long vox_max_item;    // samples of the level's largest item (statistics)
+  unsigned long long border_used;     // weighted mode: entries of the level's border lists
   unsigned int error;                 // nonzero: a kernel detected a problem
   unsigned int units;                 // voxel partition units queued this level
   unsigned int unit_head;             // units taken by the partition kernel

@@ -57,10 +57,6 @@ struct Workspace {
   };
   std::vector<Block> blocks;
   bool busy = false;
-  // dense grids of the weighted mode (Section 4.2.4): zeroed when
-  // allocated, and every launch leaves the cells it touched empty again
-  void* wgrid = nullptr;
-  size_t wgrid_bytes = 0;
   int take(size_t b) {
     int best = -1;
     for (size_t i = 0; i < blocks.size(); ++i)
@@ -485,7 +481,7 @@ uint64_t workspace_bytes(cudaStream_t st) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
   auto it = g_ws.find({dev, st});
   if (it == g_ws.end() || !it->second) return 0;
-  uint64_t b = it->second->wgrid_bytes;
+  uint64_t b = 0;
   for (auto& k : it->second->blocks) b += k.p ? k.bytes : 0;
   return b;
 }
@@ -504,7 +500,6 @@ void release_workspace(cudaStream_t st) {
   }
   for (auto& k : w->blocks)
     if (k.p) cudaFree(k.p);
-  if (w->wgrid) cudaFree(w->wgrid);
   delete w;
 }
 
@@ -628,11 +623,12 @@ uint64_t estimate_build_bytes(uint64_t n, const lod_params_t& p) {
   const uint64_t pool = (2 * pyr_size(d) + ipow8(d) + ipow8(d) / 32 + 1) * 4;
   const uint64_t nodes = 64 + 16 * ((n + T - 1) / T);
   // result + one refinement buffer + two staging levels of one record per
-  // point (plus exact sums when filtering) + the voxel array's first
+  // point (plus exact sums when filtering, plus the border lists when
+  // weighting) + the voxel array's first
   // estimate + node aux + pool, plus the 32-byte leaf staging of modes that
   // keep input indices
   const bool keep_idx = keeps_index(p);
-  const uint64_t staging = n * (p.mode == LOD_FILTER ? 64 : 32);
+  const uint64_t staging = n * (p.mode == LOD_FILTER ? 64 : (p.mode == LOD_WEIGHTED ? 48 : 32));
   return estimate_result_bytes(n, p) + n * 20 + staging + n * 8 + (keep_idx ? n * 32 : 0) +
          nodes * sizeof(NodeAux) + pool + (16u << 20);
 }
@@ -1166,37 +1162,20 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       LOD_CK(d_sum1.alloc(stage_cap * 16));
     }
   }
-  // weighted mode: one dense grid per persistent CTA
+  // weighted mode: the border lists of one level (no more entries than the
+  // level's items have samples)
   const bool weighted = prm.mode == LOD_WEIGHTED;
-  const int wctas = sm_count();
-  const size_t cells = size_t(1) << 21;
-  DevBuf d_wtmp(st);
-  unsigned char* wbase = nullptr;
+  DevBuf d_border(st, ws), d_blist(st, ws);
+  uint64_t border_cap = 0;
   if (weighted && n_vlev > 0) {
-    const size_t wbytes = (size_t)wctas * wgrid_bytes_per_cta();
-    const size_t wzero = (size_t)wctas * cells * 36;  // sums and counts start at zero; the lists need not
-    if (ws) {
-      if (ws->wgrid_bytes < wbytes) {
-        if (ws->wgrid) {
-          LOD_CK(cudaStreamSynchronize(st));
-          cudaFree(ws->wgrid);
-          ws->wgrid = nullptr;
-          ws->wgrid_bytes = 0;
-        }
-        LOD_CK(cudaMalloc(&ws->wgrid, wbytes));
-        ws->wgrid_bytes = wbytes;
-        LOD_CK(cudaMemsetAsync(ws->wgrid, 0, wzero, st));
-      }
-      wbase = static_cast<unsigned char*>(ws->wgrid);
-    } else {
-      LOD_CK(d_wtmp.alloc(wbytes));
-      LOD_CK(cudaMemsetAsync(d_wtmp.p, 0, wzero, st));
-      wbase = d_wtmp.as<unsigned char>();
-    }
+    for (int l = 0; l < n_vlev; ++l)
+      border_cap = std::max<uint64_t>(border_cap, leaf_cap[kMaxLevels + 1 + l + 1] + leaf_cap[l + 1]);
+    LOD_CK(d_border.alloc(total_cap * sizeof(uint4)));
+    LOD_CK(d_blist.alloc(border_cap * sizeof(int4)));
   }
   const uint32_t units_cap = (uint32_t)std::min<uint64_t>((uint64_t)max_items * 64, 1u << 20);
   LOD_CK(d_units.alloc((size_t)units_cap * sizeof(uint4)));
-  if (!weighted) LOD_CK(d_order.alloc((size_t)max_items * 4));
+  LOD_CK(d_order.alloc((size_t)max_items * 4));
   const size_t lctr_bytes = (size_t)std::max(n_vlev, 1) * sizeof(DevCounters);
   LOD_CK(d_lctr.alloc(lctr_bytes));
   LOD_CK(d_vstate.alloc(2 * sizeof(unsigned long long)));
@@ -1258,22 +1237,18 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       vl.n_parents = n_par;
       // the deepest level takes its items in node order; every level scan
       // orders the items of the level above, larger ones first
-      vl.order = (l == n_vlev - 1 || weighted) ? nullptr : d_order.as<uint32_t>();
-      vl.next_order = (l == 0 || weighted) ? nullptr : d_order.as<uint32_t>();
+      vl.order = l == n_vlev - 1 ? nullptr : d_order.as<uint32_t>();
+      vl.next_order = l == 0 ? nullptr : d_order.as<uint32_t>();
       {
         const uint32_t q = g_tune_queue_ranges.load();
         vl.queue_ranges = q == 0 ? 4u : (q == 1 ? 0xFFFFFFFFu : q);
         vl.range_cells = g_tune_range_cells.load();
       }
-      if (weighted) {
-        vl.wgrid = reinterpret_cast<unsigned long long*>(wbase);
-        vl.wcnt = reinterpret_cast<uint32_t*>(wbase + (size_t)wctas * cells * 32);
-        vl.wtouch = reinterpret_cast<uint32_t*>(wbase + (size_t)wctas * cells * 36);
-        LOD_LAUNCH(debug_stats() ? kVoxLevelNames[l] : "voxelize", 0,
-                   launch_wvox(A, vl, lc, (int)std::min<uint32_t>((uint32_t)wctas, n_par), vst));
-      } else {
-        LOD_LAUNCH(debug_stats() ? kVoxLevelNames[l] : "voxelize", 0, launch_vox(A, vl, lc, vst));
-      }
+      vl.border = d_border.as<uint4>();
+      vl.border_list = d_blist.as<int4>();
+      vl.border_cap = border_cap;
+      if (weighted) LOD_LAUNCH("weighted_border", 0, launch_wborder(A, vl, lc, vst));
+      LOD_LAUNCH(debug_stats() ? kVoxLevelNames[l] : "voxelize", 0, launch_vox(A, vl, lc, vst));
       vox_rec[l] = prof.recs.size();
       LOD_LAUNCH("level_scan", 0,
                  launch_level_scan(A, vl, d_pref.as<uint32_t>() + (size_t)l * pstride + (nt + 1), n_par,

@@ -42,6 +42,7 @@
 // reads them (so each record is read once).
 #include "common.cuh"
 #include "kernels.h"
+#include "wgrid.cuh"
 
 namespace lodk {
 
@@ -77,6 +78,7 @@ constexpr uint32_t kCapLeaf = kDenseBytes / 10;    // filtered leaf, <= 65535 po
 constexpr uint32_t kCapNarrow = kDenseBytes / 18;  // filtered, 32-bit sums: R, G, B, n
 constexpr uint32_t kCapWide = kDenseBytes / 30;    // filtered, 64-bit sums: R, G, B (low and high words), n
 constexpr uint32_t kCapPick = kDenseBytes / 22;    // single sample: u64 {key high word, index}, {index, rgba}, n
+constexpr uint32_t kCapWeighted = kDenseBytes / 38;  // weighted: w R, w G, w B, w (low and high words), n
 constexpr uint64_t kNarrowMaxSamples = 0xFFFFFFFFull / 255;  // 32-bit channel sums cannot overflow
 constexpr uint64_t kLeafMaxSamples = 0xFFFFu;                // a 16-bit count cannot
 constexpr uint64_t kMask40 = (1ull << 40) - 1;
@@ -216,6 +218,8 @@ struct VoxShared {
   int32_t cmin[3];             // header: the child's min corner
   uint32_t n_wraps;            // 16-bit field wraps listed by the pass
   unsigned long long cparent, cfirst;  // header: parent node, first child (absolute)
+  unsigned long long nbase;    // header: the tile's first node
+  unsigned long long pfirst;   // header: the parent's first child (absolute)
   unsigned long long pbase;    // header: the child's first leaf point (absolute)
   uint32_t cpre[9];            // inner items: prefix of the children's record counts
   uint32_t settle;             // single sample: the pass needs settle_pick
@@ -223,6 +227,8 @@ struct VoxShared {
   unsigned long long cdense[8];  // ... their places in the voxel array
   uint32_t wsum[kVoxWarps];
   uint32_t qbase[4];           // rank of the first cell of each quarter of the octant
+  uint4 border[8];             // weighted: the border lists of the parent's children, in octant order
+  uint32_t pmask;              // ... and which octants they are
   uint32_t pick_level, idx_bound;  // header: level of the parent, bound of the tile's input indices
   uint32_t next;               // the item or unit taken next
   ItemInfo I;
@@ -265,11 +271,11 @@ __device__ __forceinline__ uint16_t* vox_cells() {
   return reinterpret_cast<uint16_t*>(vox_fields() + WORDS * CAP);
 }
 
-// Empty dense entries: all zero bytes in filtered mode (whatever the
+// Empty dense entries: all zero bytes in the averaging modes (whatever the
 // layout), ~0 keys and zero counts in the single-sample modes.
 template <int MODE>
 __device__ __forceinline__ void vox_clear_dense() {
-  if (MODE == LOD_FILTER) {
+  if (MODE == LOD_FILTER || MODE == LOD_WEIGHTED) {
     uint4* z = reinterpret_cast<uint4*>(vox_smem + kDenseOff);
     for (uint32_t i = threadIdx.x; i < kDenseBytes / 16u; i += kVoxThreads) z[i] = make_uint4(0, 0, 0, 0);
   } else {
@@ -729,6 +735,89 @@ __device__ __noinline__ void settle_pick(PickArgs P, const int4* src, const uint
   if (threadIdx.x == 0) S.settle = 0;
 }
 
+// Neighbourhood-weighted average (Section 4.2.4; see k_weighted.cu): a sample
+// adds its weight and weighted colours to those of its 2x2x2 cells that lie in
+// the item's octant, are occupied and have a rank of the pass.  Sums are exact
+// 64-bit integers in low and high words (a weighted colour has at most 32
+// bits, so the high word only counts the low word's wraps).
+__device__ __forceinline__ void add_weighted(const WBlock& b, uint32_t rgba, const uint32_t* qbase, uint32_t lo, uint32_t span) {
+  const ItemInfo& I = vox_shared().I;
+  const uint32_t oct[3] = {I.kx, I.ky, I.kz};
+  float sq[3][2];
+  bool in[3][2];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float e1 = __fsub_rn(b.e0[a], 1.0f);
+    sq[a][0] = __fmul_rn(b.e0[a], b.e0[a]);
+    sq[a][1] = __fmul_rn(e1, e1);
+    in[a][0] = ((b.j1[a] - 1) >> 6) == (int32_t)oct[a];
+    in[a][1] = (b.j1[a] >> 6) == (int32_t)oct[a];
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int kx = (k >> 2) & 1, ky = (k >> 1) & 1, kz = k & 1;
+    if (!(in[0][kx] && in[1][ky] && in[2][kz])) continue;
+    const uint32_t w = w_weight(__fadd_rn(__fadd_rn(sq[0][kx], sq[1][ky]), sq[2][kz]));
+    if (!w) continue;
+    const uint32_t cell = ((uint32_t)(b.j1[0] - 1 + kx) & 63u) | (((uint32_t)(b.j1[1] - 1 + ky) & 63u) << 6) |
+                          (((uint32_t)(b.j1[2] - 1 + kz) & 63u) << 12);
+    const uint32_t word = vox_bits()[cell >> 5], bit = cell & 31u;
+    if (!((word >> bit) & 1u)) continue;
+    const uint32_t rk = vox_wrank()[cell >> 5] + (qbase ? qbase[cell >> 16] : 0u) + __popc(word & ((1u << bit) - 1u)) - lo;
+    if (rk >= span) continue;
+    uint32_t* const F = vox_fields() + rk;
+    const uint32_t v[4] = {w * (rgba & 255u), w * ((rgba >> 8) & 255u), w * ((rgba >> 16) & 255u), w};
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const uint32_t old = atomicAdd(F + 2u * f * kCapWeighted, v[f]);
+      if (old + v[f] < old) atomicAdd(F + (2u * f + 1u) * kCapWeighted, 1u);
+    }
+  }
+}
+
+// The sample's own cell takes its count.
+__device__ __forceinline__ void add_weighted_own(uint32_t cell, uint32_t n, const uint32_t* qbase, uint32_t lo, uint32_t span) {
+  const uint32_t word = vox_bits()[cell >> 5];
+  const uint32_t rk = vox_wrank()[cell >> 5] + (qbase ? qbase[cell >> 16] : 0u) + __popc(word & ((1u << (cell & 31u)) - 1u)) - lo;
+  if (rk < span && atomicAdd(vox_fields() + 8u * kCapWeighted + rk, n) == 0u) vox_cells<9, kCapWeighted>()[rk] = (uint16_t)cell;
+}
+
+// Pass 2 of the weighted mode: the item's own samples, then its siblings'
+// border lists.  Issue-bound (up to eight weights a sample), so the samples
+// are taken one at a time.
+__device__ __forceinline__ void acc_weighted(const int4* src, const int4* border_list, bool leaf, uint32_t total, uint32_t lo,
+                                             uint32_t span) {
+  VoxShared& S = vox_shared();
+  const uint32_t* const qbase = S.D > 0xFFFFu ? S.qbase : nullptr;
+  const CellMap cm(S.I);
+  const uint32_t oct = (S.I.kx << 2) | (S.I.ky << 1) | S.I.kz;
+  uint32_t ci = 0;
+  for (uint32_t i = threadIdx.x; i < total; i += kVoxThreads) {
+    if (leaf) {
+      const int4 q = __ldcg(src + i);
+      add_weighted_own(cm(q), 1u, qbase, lo, span);
+      add_weighted(w_point_block(q, S.I.pmin, S.I.Lp), (uint32_t)q.w, qbase, lo, span);
+    } else {
+      const int4 q = __ldcg(src + child_record(S, i, ci));
+      add_weighted_own(voxel_cell((uint32_t)q.x), (uint32_t)q.z, qbase, lo, span);
+      add_weighted(w_voxel_block((uint32_t)q.x, oct), (uint32_t)q.y, qbase, lo, span);
+    }
+    if (total - i <= kVoxThreads) break;  // (i + kVoxThreads may not fit 32 bits)
+  }
+  for (uint32_t k = 0, r = 0; k < 8; ++k) {
+    if (!((S.pmask >> k) & 1u)) continue;
+    const uint4 L = S.border[r++];
+    if (k == oct) continue;
+    const int4* const e = border_list + (L.x | ((uint64_t)L.y << 32));
+    for (uint32_t i = threadIdx.x; i < L.z; i += kVoxThreads) {
+      const int4 q = __ldcg(e + i);
+      if (L.w) add_weighted(w_point_block(q, S.I.pmin, S.I.Lp), (uint32_t)q.w, qbase, lo, span);
+      else add_weighted(w_voxel_block((uint32_t)q.x & 0x1FFFFFu, k), (uint32_t)q.y, qbase, lo, span);
+      if (L.z - i <= kVoxThreads) break;
+    }
+  }
+}
+
 // The cell of rank r (its lower 16 bits are kept beside the entry): the
 // upper two bits are the quarter of the octant the rank lies in.
 __device__ __forceinline__ uint32_t rank_cell(const VoxShared& S, uint32_t low, uint32_t r) {
@@ -795,6 +884,23 @@ __device__ __forceinline__ void extract_sums(int4* stage_out, ulonglong2* sums_o
   }
 }
 
+// Extraction of the weighted mode.
+__device__ __forceinline__ void extract_weighted(int4* stage_out, uint64_t stage_cap, uint64_t at, uint32_t lo, uint32_t span) {
+  VoxShared& S = vox_shared();
+  uint32_t* const F = vox_fields();
+  uint16_t* const K = vox_cells<9, kCapWeighted>();
+  for (uint32_t i = threadIdx.x; i < span; i += kVoxThreads) {
+    const uint32_t cell = rank_cell(S, K[i], lo + i), n = F[8u * kCapWeighted + i];
+    unsigned long long s[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) s[f] = F[2u * f * kCapWeighted + i] | ((unsigned long long)F[(2u * f + 1u) * kCapWeighted + i] << 32);
+#pragma unroll
+    for (uint32_t f = 0; f < 9u; ++f) F[f * kCapWeighted + i] = 0u;
+    const uint32_t rgba = w_round(s[0], s[3]) | (w_round(s[1], s[3]) << 8) | (w_round(s[2], s[3]) << 16) | 0xFF000000u;
+    if (at + i < stage_cap) stage_out[at + i] = make_int4((int)parent_cell(cell, S.I), (int)rgba, (int)n, (int)kNone);
+  }
+}
+
 // Extraction of the single-sample modes.
 template <int MODE>
 __device__ __forceinline__ void extract_pick(const PickArgs& P) {
@@ -851,6 +957,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       S.I.leaf = (c.flags & LOD_NODE_LEAF) != 0;
       S.I.n = S.I.leaf ? c.point_count : c.voxel_count;
       S.I.npts = c.point_count;
+      S.nbase = td.node_base;
       S.cparent = td.node_base + c.parent;
       S.cfirst = td.node_base + c.first_child;
       S.pbase = td.pt_base + c.point_offset;
@@ -872,6 +979,8 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
     if (lane == 8) {
       const lod_node_t p = v.nodes[S.cparent];
       S.I.Lp = p.log2_size;
+      S.pmask = p.child_mask;
+      S.pfirst = S.nbase + p.first_child;
       S.I.pmin[0] = p.min[0];
       S.I.pmin[1] = p.min[1];
       S.I.pmin[2] = p.min[2];
@@ -902,7 +1011,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
 #pragma unroll
   for (uint32_t i = 0; i < kWords / 4u / kVoxThreads; ++i) bits4[tid + i * kVoxThreads] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  constexpr bool PICKLIKE = MODE != LOD_FILTER;  // one sample kept per cell
+  constexpr bool WEIGHTED = MODE == LOD_WEIGHTED, PICKLIKE = MODE != LOD_FILTER && !WEIGHTED;  // one sample kept per cell
   const bool leaf = S.I.leaf;
   const bool lead = r_unit == 0;  // the one CTA of the item that publishes the children's voxels
   // the units of an item split up front run side by side, so each of them
@@ -913,8 +1022,10 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
   uint32_t next_k = 0;
   if (next_item && tid == 0) next_k = atomicAdd(&ctr->item_head, 1u);
 
+  if (WEIGHTED && tid < (uint32_t)__popc(S.pmask)) S.border[tid] = v.border[S.pfirst + tid];
+
   // ---- pass 1: mark the occupied cells
-  if (!leaf) mark_inner<!PICKLIKE>(v.stage_in, total, lead ? v.dense : nullptr, v.dense_cap);
+  if (!leaf) mark_inner<MODE == LOD_FILTER>(v.stage_in, total, lead ? v.dense : nullptr, v.dense_cap);
   else if (a.wide) mark_wide(a.wide + 2 * S.pbase, total, own_leaf ? a.out + S.pbase : nullptr, own_leaf ? a.out_idx + S.pbase : nullptr);
   else mark_leaf(a.out + S.pbase, total);
   __syncthreads();
@@ -966,7 +1077,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
   }
   // the narrowest sums that provably cannot overflow for the points of this cube
   const SumLayout lay = leaf && S.I.npts <= kLeafMaxSamples ? kLeaf16 : (S.I.npts <= kNarrowMaxSamples ? kNarrow : kWide);
-  const uint32_t cap = PICKLIKE ? kCapPick : (lay == kLeaf16 ? kCapLeaf : (lay == kNarrow ? kCapNarrow : kCapWide));
+  const uint32_t cap = PICKLIKE ? kCapPick : WEIGHTED ? kCapWeighted : (lay == kLeaf16 ? kCapLeaf : (lay == kNarrow ? kCapNarrow : kCapWide));
   const uint32_t C = (v.range_cells && v.range_cells < cap) ? v.range_cells : cap;  // ranks per pass
   // thread 0: the item's first staging record.  The reservation (or, for
   // a unit, the read of the first attempt's) is issued here and its value
@@ -1019,6 +1130,8 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       P.out_at = 0;
       if (!leaf) pick_inner<MODE>(P, src, total);
       else pick_leaf<MODE>(P, src, pidx, total);
+    } else if (WEIGHTED) {
+      acc_weighted(src, v.border_list, leaf, total, lo, span);
     } else if (leaf) {
       if (lay == kLeaf16) acc_leaf16(src, total, lo, span);
       else if (lay == kNarrow) acc_leaf_sums<false>(src, total, lo, span);
@@ -1035,6 +1148,8 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       extract_pick<MODE>(P);
       __syncthreads();
       if (S.settle) settle_pick<MODE>(P, src, pidx, leaf, total);
+    } else if (WEIGHTED) {
+      extract_weighted(v.stage_out, v.stage_cap, at, lo, span);
     } else if (lay == kLeaf16) {
       extract_sums<kLeaf16>(v.stage_out, v.stage_out_sum, v.stage_cap, at, lo, span);
     } else if (lay == kNarrow) {
@@ -1043,7 +1158,7 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       extract_sums<kWide>(v.stage_out, v.stage_out_sum, v.stage_cap, at, lo, span);
     }
     __syncthreads();
-    if (!PICKLIKE && lay == kLeaf16 && r1 - lo > C) {  // more passes follow: they list their own wraps
+    if (MODE == LOD_FILTER && lay == kLeaf16 && r1 - lo > C) {  // more passes follow: they list their own wraps
       if (tid == 0) S.n_wraps = 0;
       __syncthreads();
     }
@@ -1139,6 +1254,7 @@ int vox_init() {
     vox_attrs<LOD_PICK>();
     vox_attrs<LOD_FIRST>();
     vox_attrs<LOD_RANDOM>();
+    vox_attrs<LOD_WEIGHTED>();
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
@@ -1172,6 +1288,7 @@ cudaError_t launch_vox(const BuildArgs& a, const VoxLevel& v, DevCounters* ctr, 
     case LOD_PICK: return launch_vox_mode<LOD_PICK>(a, v, ctr, st);
     case LOD_FIRST: return launch_vox_mode<LOD_FIRST>(a, v, ctr, st);
     case LOD_RANDOM: return launch_vox_mode<LOD_RANDOM>(a, v, ctr, st);
+    case LOD_WEIGHTED: return launch_vox_mode<LOD_WEIGHTED>(a, v, ctr, st);
     default: return launch_vox_mode<LOD_FILTER>(a, v, ctr, st);
   }
 }

@@ -1,7 +1,7 @@
-// Dense-grid accumulation shared by the neighbourhood-weighted voxel pass
-// (Section 4.2.4) and the merge of out-of-core chunks: per grid cell one
-// 32-byte sector of four 64-bit sums, a 32-bit count, and a list of the
-// cells touched since the grid was last emptied.  Internal.
+// Neighbourhood weights (Section 4.2.4), for the weighted voxel pass and the
+// merge of out-of-core chunks, and the merge's dense-grid accumulation: per
+// grid cell one 32-byte sector of four 64-bit sums, a 32-bit count, and a
+// list of the cells touched since the grid was last emptied.  Internal.
 #pragma once
 
 #include "common.cuh"
@@ -10,6 +10,61 @@ namespace lodk {
 
 constexpr uint32_t kGridCells = 1u << 21;  // 128^3
 constexpr float kWScale = 16777216.0f;     // 2^24: fixed-point weight unit
+
+// The 2x2x2 cells a sample reaches and its offsets from their centres: per
+// axis the cells j1 - 1 and j1 of the 128^3 grid (j1 - 1 may be -1 and j1 128:
+// outside the grid), j1 = floor(pos - 1/2) + 1, the offset e0 = pos - (j1 -
+// 1/2) from the first one's centre and e0 - 1 from the second's, in cells.
+struct WBlock {
+  int32_t j1[3];
+  float e0[3];
+};
+
+// Of a point of a node with min corner mn and edge 2^L: pos = d 2^(7-L).  With
+// s = L - 7 > 0, pos - 1/2 = (d - 2^(s-1)) / 2^s: the offset is the remainder
+// m < 2^s (at most 25 bits, rounded once to single precision) over 2^s.  For
+// L <= 7 a point is a cell corner, half a cell from the centres around it.
+__device__ __forceinline__ WBlock w_point_block(const int4& q, const int32_t (&mn)[3], uint32_t L) {
+  const uint32_t d[3] = {(uint32_t)q.x - (uint32_t)mn[0], (uint32_t)q.y - (uint32_t)mn[1],
+                         (uint32_t)q.z - (uint32_t)mn[2]};
+  WBlock b;
+  if (L > 7) {
+    const uint32_t s = L - 7, half = 1u << (s - 1), mask = (half << 1) - 1u;
+    const float inv = __int_as_float((int)(127u - s) << 23);  // 2^-s
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      b.j1[a] = (int32_t)((d[a] >> s) + ((d[a] & mask) >= half ? 1u : 0u));
+      b.e0[a] = __fmul_rn(__uint2float_rn((d[a] + half) & mask), inv);
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      b.j1[a] = (int32_t)(d[a] << (7 - L));
+      b.e0[a] = 0.5f;
+    }
+  }
+  return b;
+}
+
+// Of a voxel (cell q of the child in octant k) at its centre: pos = 64 b + (q +
+// 1/2) / 2, a quarter of a cell from its parent cell's centre.
+__device__ __forceinline__ WBlock w_voxel_block(uint32_t cell, uint32_t k) {
+  const uint32_t q[3] = {cell & 127u, (cell >> 7) & 127u, cell >> 14};
+  WBlock b;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    b.j1[a] = (int32_t)(64u * ((k >> (2 - a)) & 1u) + ((q[a] + 1u) >> 1));
+    b.e0[a] = (q[a] & 1u) ? 0.25f : 0.75f;
+  }
+  return b;
+}
+
+// Weight at squared distance d2: 1 - sqrt(d2) in single precision (each
+// operation rounded on its own), as a multiple of 2^-24 (ties to even); 0 at
+// a distance of 1 and beyond.
+__device__ __forceinline__ uint32_t w_weight(float d2) {
+  return d2 < 1.0f ? __float2uint_rn(__fmul_rn(__fsub_rn(1.0f, __fsqrt_rn(d2)), kWScale)) : 0u;
+}
 
 // One weighted contribution to grid cell `cell`: the first toucher (the
 // weight sum was zero before) lists the cell for extraction.

@@ -98,3 +98,24 @@ def test_ranks_beyond_16_bits(lod, mode):
     pts[:, :3] = rng.integers(0, 1 << 14, (1_600_000, 3))
     pts[:, 3] = rng.integers(-(2**31), 2**31, 1_600_000)
     check(lod, pts, 300_000, mode, max_depth=1)
+
+
+@pytest.mark.parametrize("depth", [1, 2, 3])
+@pytest.mark.parametrize("L", [2, 6, 7, 8, 9, 15, 31, 32])
+def test_weighted_samples_across_octants(lod, L, depth):
+    # points within two cells of the middle planes of a cube of edge 2^L, on
+    # one, two or all three axes: their weights reach one to seven siblings;
+    # deeper trees hand voxels across the planes as well
+    rng = np.random.default_rng(100 * L + depth)
+    n, mid, cell = 3000, 1 << (L - 1), max(1, (1 << L) >> 7)
+    p = rng.integers(0, 1 << L, (n, 3))
+    near = rng.random((n, 3)) < 0.6
+    p = np.where(near, mid + rng.integers(-2 * cell, 2 * cell + 1, (n, 3)), p)
+    p[:3] = mid
+    p[3:6] = mid - 1
+    p[6:8] = [[0, 0, 0], [(1 << L) - 1] * 3]
+    p = np.clip(p, 0, (1 << L) - 1) - (1 << 31 if L == 32 else 0)
+    pts = np.empty((n, 4), np.int32)
+    pts[:, :3] = p
+    pts[:, 3] = rng.integers(-(2**31), 2**31, n)
+    check(lod, pts, 20, 2, max_depth=depth)
