@@ -253,7 +253,8 @@ const char* lod_error_string(int status);
  * pool, which the library sets to keep freed memory for reuse.  The paper
  * has no counterpart (its buffers are allocated once, Section 4.1.6).
  * lod_scratch_bytes: device bytes the workspace of `stream` holds now.
- * lod_trim: waits for `stream` to finish its work, frees its workspace and
+ * lod_trim: waits for `stream` to finish its work, frees its workspace and the
+ *   calling thread's page-locked upload memory (at most 8 MB per thread), and
  *   returns the pool's unused memory to the device.  Results stay valid;
  *   the next build on the stream allocates its scratch again.  A workspace
  *   that a build on another thread is using at that moment is left alone.

@@ -269,6 +269,7 @@ int lod_trim(void* stream) {
   cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return to_status(e);
   lodk::release_workspace(st);
+  lodk::release_thread_arena();
   int dev = 0;
   cudaMemPool_t pool;
   if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)

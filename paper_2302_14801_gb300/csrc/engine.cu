@@ -216,39 +216,56 @@ struct HostStage {
 };
 thread_local HostStage tl_stage;
 
-// Pinned host arena for small uploads: cudaMemcpyAsync from pageable memory
-// synchronises the stream, from pinned memory it does not.  The arena is
-// recycled at every host synchronisation of the build (all earlier copies
-// have completed by then).
+// Pinned host memory for small uploads: cudaMemcpyAsync from pageable memory
+// synchronises the stream, from pinned memory it does not.  One arena per
+// host thread, kept between its builds up to kArenaKeep bytes (allocating and
+// freeing page-locked memory took 0.2 ms of every build, and the free waits
+// for the whole device, other threads' builds included); given back by
+// lod_trim and when the thread ends.
+constexpr size_t kArenaKeep = 8u << 20;
+struct PinnedArena {
+  char* base = nullptr;
+  size_t cap = 0;
+  ~PinnedArena() { release(); }
+  void release() {
+    if (base) cudaFreeHost(base);
+    base = nullptr;
+    cap = 0;
+  }
+};
+thread_local PinnedArena tl_arena;
+
+// The uploads of one build through its thread's arena, which is recycled at
+// every host synchronisation of the build (all earlier copies have completed
+// by then).  A build waits for its stream before it gives the arena back.
 struct Uploader {
   cudaStream_t st;
-  char* base = nullptr;
-  size_t cap = 0, used = 0;
+  PinnedArena& ar;
+  size_t used = 0;
   std::vector<char*> retired;
-  explicit Uploader(cudaStream_t s) : st(s) {}
+  explicit Uploader(cudaStream_t s) : st(s), ar(tl_arena) {}
+  Uploader(const Uploader&) = delete;
   ~Uploader() {
     cudaStreamSynchronize(st);
     for (char* r : retired) cudaFreeHost(r);
-    if (base) cudaFreeHost(base);
+    if (ar.cap > kArenaKeep) ar.release();
   }
   cudaError_t put(void* dst, const void* src, size_t bytes) {
     if (!bytes) return cudaSuccess;
     const size_t need = (bytes + 255) & ~size_t(255);
-    if (used + need > cap) {
-      if (base) retired.push_back(base);
-      cap = std::max<size_t>(need, std::max<size_t>(cap * 2, 1 << 20));
+    if (used + need > ar.cap) {
+      const size_t cap = std::max<size_t>(need, std::max<size_t>(ar.cap * 2, 1 << 20));
+      if (ar.base) retired.push_back(ar.base);
+      ar.base = nullptr;
+      ar.cap = used = 0;
       void* q = nullptr;
-      cudaError_t e = cudaMallocHost(&q, cap);
-      if (e != cudaSuccess) {
-        base = nullptr;
-        cap = used = 0;
-        return e;
-      }
-      base = static_cast<char*>(q);
-      used = 0;
+      const cudaError_t e = cudaMallocHost(&q, cap);
+      if (e != cudaSuccess) return e;
+      ar.base = static_cast<char*>(q);
+      ar.cap = cap;
     }
-    std::memcpy(base + used, src, bytes);
-    cudaError_t e = cudaMemcpyAsync(dst, base + used, bytes, cudaMemcpyHostToDevice, st);
+    std::memcpy(ar.base + used, src, bytes);
+    cudaError_t e = cudaMemcpyAsync(dst, ar.base + used, bytes, cudaMemcpyHostToDevice, st);
     used += need;
     return e;
   }
@@ -504,6 +521,8 @@ void release_workspace(cudaStream_t st) {
 }
 
 
+void release_thread_arena() { tl_arena.release(); }
+
 uint32_t default_root_depth(uint64_t n, uint32_t T, uint32_t max_depth) {
   if (n <= T || max_depth == 0 || T == 0) return 0;
   uint32_t d = ceil_log4((double)n / (double)T) + 1;
@@ -756,53 +775,111 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   } while (0)
 
   DevBuf d_points(st), d_index(st);  // results
-  DevBuf d_tiles(st, ws), d_chunk0(st, ws), d_chunk_src(st, ws), d_bbox(st, ws), d_ctr(st, ws), d_nchunks(st, ws);
   LOD_CK(d_points.alloc(M * 16));
   if (want_idx) LOD_CK(d_index.alloc(M * 4));
-  LOD_CK(d_tiles.alloc(nt * sizeof(TileDesc)));
-  LOD_CK(d_chunk0.alloc((nt + 1) * sizeof(uint64_t)));
-  LOD_CK(d_chunk_src.alloc(std::max<uint64_t>(n_chunks0, 1) * 4));
-  LOD_CK(d_bbox.alloc(nt * 6 * sizeof(int)));
-  LOD_CK(d_ctr.alloc(sizeof(DevCounters)));
-  LOD_CK(d_nchunks.alloc(sizeof(unsigned long long)));
-  LOD_CK(cudaMemsetAsync(d_ctr.p, 0, sizeof(DevCounters), st));
-  LOD_CK(up_.put(d_tiles.p, td.data(), nt * sizeof(TileDesc)));
-  LOD_CK(up_.put(d_chunk0.p, chunk0.data(), (nt + 1) * sizeof(uint64_t)));
-  if (n_chunks0)
-    LOD_CK(up_.put(d_chunk_src.p, chunk_tile.data(), n_chunks0 * 4));
-  {
-    std::vector<int> init(6 * nt);
-    for (uint32_t t = 0; t < nt; ++t)
-      for (int i = 0; i < 3; ++i) {
-        init[6 * t + i] = INT_MAX;
-        init[6 * t + 3 + i] = INT_MIN;
-      }
-    LOD_CK(up_.put(d_bbox.p, init.data(), init.size() * sizeof(int)));
-  }
-
-  // ---- bounding box (root cube)
-  LOD_LAUNCH("bbox", 16.0 * M,
-             launch_bbox(d_tiles.as<TileDesc>(), d_chunk_src.as<uint32_t>(), n_chunks0, d_chunk0.as<uint64_t>(),
-                         d_bbox.as<int>(), grid, st));
-  std::vector<int> bbox(6 * nt);
-  DevBuf d_abort(st, ws);
-  if (sync_roots) {
-    LOD_CK(cudaMemcpyAsync(bbox.data(), d_bbox.p, bbox.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
-    LOD_CK(cudaStreamSynchronize(st));
-    clk.tick("bbox");
-    up_.recycle();
-    prof.resolve();
-    ++S.host_syncs;
-  } else {
-    LOD_CK(d_abort.alloc(sizeof(unsigned int)));
-    LOD_CK(cudaMemsetAsync(d_abort.p, 0, sizeof(unsigned int), st));
-  }
-
+  // node capacity and place of every tile (the node pass doubles back with
+  // larger ones if a tile needs more)
+  std::vector<uint32_t> node_cap(nt);
+  uint64_t total_cap = 0;
+  auto place_nodes = [&] {
+    total_cap = 0;
+    for (uint32_t t = 0; t < nt; ++t) {
+      td[t].node_base = total_cap;
+      td[t].node_cap = node_cap[t];
+      total_cap += node_cap[t];
+    }
+  };
+  for (uint32_t t = 0; t < nt; ++t) node_cap[t] = (uint32_t)std::min<uint64_t>(64 + 16 * ((td[t].n + T - 1) / T), 0x7FFFFFFFull);
+  place_nodes();
+  // The build's small inputs lie in one device block, so that a build without
+  // refinement uploads them with one copy: tile table, chunk space, box
+  // accumulators, chunk count, then (when the first round needs no box from
+  // the host) its pyramid jobs and counting grids.
   std::vector<SrcDesc> srcs(nt);
   uint64_t src_bound0 = 0;
-  for (uint32_t t = 0; t < nt; ++t) {
-    if (!sync_roots) {
-      // cube unknown yet (set on the device); depth from the counts alone
+  for (uint32_t t = 0; t < nt; ++t) src_bound0 += td[t].n / (T + 1ull);
+  uint64_t src_cap = nt + src_bound0 + 16;
+  size_t in_bytes = 0;
+  auto section = [&](size_t bytes) {
+    const size_t o = in_bytes;
+    in_bytes = (in_bytes + bytes + 255) & ~size_t(255);
+    return o;
+  };
+  const size_t o_tiles = section(nt * sizeof(TileDesc)), o_chunk0 = section((nt + 1) * sizeof(uint64_t)),
+               o_bbox = section(nt * 6 * sizeof(int)), o_nchunks = section(sizeof(unsigned long long)),
+               o_chunk_src = section(std::max<uint64_t>(n_chunks0, 1) * 4);
+  std::vector<char> in_host(in_bytes);
+  std::memcpy(&in_host[o_tiles], td.data(), nt * sizeof(TileDesc));
+  std::memcpy(&in_host[o_chunk0], chunk0.data(), (nt + 1) * sizeof(uint64_t));
+  for (uint32_t t = 0; t < nt; ++t)
+    for (int i = 0; i < 3; ++i) {
+      reinterpret_cast<int*>(&in_host[o_bbox])[6 * t + i] = INT_MAX;
+      reinterpret_cast<int*>(&in_host[o_bbox])[6 * t + 3 + i] = INT_MIN;
+    }
+  std::memcpy(&in_host[o_nchunks], &n_chunks0, sizeof(n_chunks0));
+  if (n_chunks0) std::memcpy(&in_host[o_chunk_src], chunk_tile.data(), n_chunks0 * 4);
+
+  BuildArgs A;
+  std::memset(&A, 0, sizeof(A));
+
+  // ---- one counting round's grids: their pool and pyramid jobs (up passes
+  // with bottom levels d, d-4, ..., then down passes with tops 0, 4, ...)
+  std::vector<std::unique_ptr<DevBuf>> pools;
+  std::vector<PyrJob> jobs;
+  std::vector<uint32_t> up_jobs, down_jobs;  // per pass
+  PoolLayout L;
+  auto prepare_round = [&](uint32_t first, uint32_t n) -> int {
+    std::vector<uint64_t> offs;
+    L = layout_pool(srcs, first, n, &offs);
+    pools.emplace_back(new DevBuf(st, ws));
+    DevBuf& pool = *pools.back();
+    LOD_CK(pool.alloc(L.total * 4));
+    uint32_t* pb = pool.as<uint32_t>();
+    A.cnt_base = pb + L.cnt;
+    A.cursor_delta = L.start - L.cnt;
+    std::vector<std::vector<PyrJob>> up, down;
+    for (uint32_t i = 0; i < n; ++i) {
+      const uint32_t sid = first + i;
+      SrcDesc& s = srcs[sid];
+      s.ovf = pb + L.ovf + offs[4 * i + 0];
+      s.cnt = pb + L.cnt + offs[4 * i + 1];
+      s.start = pb + L.start + offs[4 * i + 2];
+      s.map = pb + L.map + offs[4 * i + 3];
+      const uint32_t d = s.d;
+      uint32_t pass = 0;
+      for (int jb = (int)d; jb > 0; jb -= 4, ++pass) {
+        if (up.size() <= pass) up.emplace_back();
+        const uint32_t k = std::min<uint32_t>(4, jb);
+        const uint64_t blocks = ipow8(jb - k);
+        for (uint64_t b = 0; b < blocks; ++b) up[pass].push_back({sid, (uint32_t)jb, (uint32_t)b});
+      }
+      pass = 0;
+      for (uint32_t jt = 0; jt < d || (d == 0 && jt == 0); jt += 4, ++pass) {
+        if (down.size() <= pass) down.emplace_back();
+        const uint64_t blocks = ipow8(jt);
+        for (uint64_t b = 0; b < blocks; ++b) down[pass].push_back({sid, jt, (uint32_t)b});
+        if (d == 0) break;
+      }
+    }
+    jobs.clear();
+    up_jobs.clear();
+    down_jobs.clear();
+    for (auto& v : up) {
+      jobs.insert(jobs.end(), v.begin(), v.end());
+      up_jobs.push_back((uint32_t)v.size());
+    }
+    for (auto& v : down) {
+      jobs.insert(jobs.end(), v.begin(), v.end());
+      down_jobs.push_back((uint32_t)v.size());
+    }
+    return LOD_OK;
+  };
+
+  // cubes still unknown (they are set on the device): the first grids'
+  // depths follow from the point counts alone
+  size_t o_jobs = 0, o_srcs = 0;
+  if (!sync_roots) {
+    for (uint32_t t = 0; t < nt; ++t) {
       SrcDesc& s = srcs[t];
       std::memset(&s, 0, sizeof(SrcDesc));
       s.tile = t;
@@ -810,9 +887,76 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       s.n = td[t].n;
       s.chunk0 = chunk0[t];
       s.priv = ipow8(s.d) > dense_max ? 1u : 0u;
-      src_bound0 += td[t].n / (T + 1ull);
-      continue;
     }
+    const int rc = prepare_round(0, nt);
+    if (rc != LOD_OK) return rc;
+    o_jobs = section(std::max<size_t>(jobs.size(), 1) * sizeof(PyrJob));
+    o_srcs = section(nt * sizeof(SrcDesc));
+    in_host.resize(in_bytes);
+    if (!jobs.empty()) std::memcpy(&in_host[o_jobs], jobs.data(), jobs.size() * sizeof(PyrJob));
+    std::memcpy(&in_host[o_srcs], srcs.data(), nt * sizeof(SrcDesc));
+  }
+  const size_t in_upload = in_bytes;
+  if (!sync_roots) in_bytes = o_srcs + src_cap * sizeof(SrcDesc);  // the grids of later rounds follow the first ones
+  DevBuf d_in(st, ws);
+  LOD_CK(d_in.alloc(in_bytes));
+  LOD_CK(up_.put(d_in.p, in_host.data(), in_upload));
+  char* const in = static_cast<char*>(d_in.p);
+  TileDesc* const g_tiles = reinterpret_cast<TileDesc*>(in + o_tiles);
+  uint64_t* const g_chunk0 = reinterpret_cast<uint64_t*>(in + o_chunk0);
+  int* const g_bbox = reinterpret_cast<int*>(in + o_bbox);
+  unsigned long long* const g_nchunks = reinterpret_cast<unsigned long long*>(in + o_nchunks);
+  uint32_t* g_chunk_src = reinterpret_cast<uint32_t*>(in + o_chunk_src);  // the round's: chunk to grid
+  DevBuf d_srcs_own(st, ws);  // the grids once they outgrow the block (or from the start when the host sets the cubes)
+  if (sync_roots) LOD_CK(d_srcs_own.alloc(src_cap * sizeof(SrcDesc)));
+  SrcDesc* g_srcs = sync_roots ? d_srcs_own.as<SrcDesc>() : reinterpret_cast<SrcDesc*>(in + o_srcs);
+
+  // Everything the host reads after the rounds, cleared and copied back as
+  // one block: the round's counters, the abort flag, per-level bounds, the
+  // node pass's counters, then per tile its node count and level starts.
+  struct NodeRead {
+    DevCounters ctr, nctr;
+    // [0, L): per level sum over all nodes of min(points, 64^3); [L, 2L): exact leaf points
+    unsigned long long leaf_cap[2 * (kMaxLevels + 1)];
+    unsigned int abort, pad;
+  };
+  const size_t rb_nn = sizeof(NodeRead), rb_lvl = rb_nn + nt * 4, rb_bytes = rb_lvl + (size_t)nt * (kMaxLevels + 1) * 4;
+  DevBuf d_rb(st, ws);
+  LOD_CK(d_rb.alloc(rb_bytes));
+  LOD_CK(cudaMemsetAsync(d_rb.p, 0, sizeof(NodeRead), st));
+  NodeRead* const g_rb = d_rb.as<NodeRead>();
+  uint32_t* const g_nn = reinterpret_cast<uint32_t*>(d_rb.as<char>() + rb_nn);
+  uint32_t* const g_lvl = reinterpret_cast<uint32_t*>(d_rb.as<char>() + rb_lvl);
+  std::vector<uint32_t> n_nodes(nt), lvl((size_t)nt * (kMaxLevels + 1));
+  std::vector<unsigned long long> leaf_cap(2 * (kMaxLevels + 1));
+  // copies the block's first `bytes` to pinned memory and waits for the stream
+  auto read_back = [&](size_t bytes, const NodeRead** out) -> int {
+    void* h = tl_stage.get(rb_bytes);
+    if (!h) return LOD_ERR_OOM;
+    LOD_CK(cudaMemcpyAsync(h, d_rb.p, bytes, cudaMemcpyDeviceToHost, st));
+    LOD_CK(cudaStreamSynchronize(st));
+    *out = static_cast<const NodeRead*>(h);
+    if (bytes == rb_bytes) {
+      std::memcpy(n_nodes.data(), static_cast<char*>(h) + rb_nn, nt * 4);
+      std::memcpy(lvl.data(), static_cast<char*>(h) + rb_lvl, lvl.size() * 4);
+      std::memcpy(leaf_cap.data(), (*out)->leaf_cap, leaf_cap.size() * 8);
+    }
+    return LOD_OK;
+  };
+
+  // ---- bounding box (root cube)
+  LOD_LAUNCH("bbox", 16.0 * M,
+             launch_bbox(g_tiles, g_chunk_src, n_chunks0, g_chunk0, g_bbox, grid, st));
+  std::vector<int> bbox(6 * nt);
+  if (sync_roots) {
+    LOD_CK(cudaMemcpyAsync(bbox.data(), g_bbox, bbox.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
+    LOD_CK(cudaStreamSynchronize(st));
+    clk.tick("bbox");
+    up_.recycle();
+    prof.resolve();
+    ++S.host_syncs;
+  }
+  for (uint32_t t = 0; sync_roots && t < nt; ++t) {
     if (tin[t].cube) {
       for (int a = 0; a < 3; ++a) td[t].min[a] = tin[t].cube[a];
       td[t].log2S = (uint32_t)tin[t].cube[3];
@@ -842,20 +986,14 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     s.n = td[t].n;
     s.chunk0 = chunk0[t];
     s.priv = ipow8(s.d) > dense_max ? 1u : 0u;  // counted through the per-CTA hash tables
-    src_bound0 += td[t].n / (T + 1ull);
   }
 
   // ---- counting rounds
-  DevBuf d_srcs(st, ws), d_jobs(st, ws), d_tmp0(st, ws), d_tmp1(st, ws), d_tmpi0(st, ws), d_tmpi1(st, ws),
+  DevBuf d_jobs(st, ws), d_chunk_src(st, ws), d_tmp0(st, ws), d_tmp1(st, ws), d_tmpi0(st, ws), d_tmpi1(st, ws),
       d_lists(st, ws), d_llen(st, ws);
   LOD_CK(d_lists.alloc((size_t)grid * kPrivSlots * sizeof(uint2)));
   LOD_CK(d_llen.alloc((size_t)grid * sizeof(uint32_t)));
-  std::vector<std::unique_ptr<DevBuf>> pools;
-  uint64_t src_cap = nt + src_bound0 + 16;
-  LOD_CK(d_srcs.alloc(src_cap * sizeof(SrcDesc)));
 
-  BuildArgs A;
-  std::memset(&A, 0, sizeof(A));
   A.n_tiles = nt;
   A.T = T;
   A.max_depth = prm.max_depth;
@@ -864,7 +1002,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   A.out_idx = want_idx ? d_index.as<uint32_t>() : nullptr;
   A.lists = d_lists.as<uint2>();
   A.list_len = d_llen.as<uint32_t>();
-  A.abort = sync_roots ? nullptr : d_abort.as<unsigned int>();
+  A.abort = sync_roots ? nullptr : &g_rb->abort;
   A.dense_max = dense_max;
   // modes that keep input indices stage each leaf point as one 32-byte record
   DevBuf d_wide(st, ws);
@@ -883,39 +1021,21 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   // scatter, before its counters are read, so that a build without
   // refinement needs no extra round trip (the table is redone if rounds
   // follow)
-  std::vector<uint32_t> node_cap(nt);
-  for (uint32_t t = 0; t < nt; ++t) node_cap[t] = (uint32_t)std::min<uint64_t>(64 + 16 * ((td[t].n + T - 1) / T), 0x7FFFFFFFull);
   DevBuf d_nodes(st);  // result
-  DevBuf d_aux(st, ws), d_lvl(st, ws), d_nn(st, ws), d_leafcap(st, ws), d_nctr(st, ws);
-  std::vector<uint32_t> n_nodes(nt), lvl((size_t)nt * (kMaxLevels + 1));
-  // [0, L): per level sum over all nodes of min(points, 64^3); [L, 2L): exact leaf points
-  std::vector<unsigned long long> leaf_cap(2 * (kMaxLevels + 1));
-  uint64_t total_cap = 0;
+  DevBuf d_aux(st, ws);
   // refined: the first round's count of refinement grids (the pass stands
   // down when it is nonzero), or null after the last round
   auto enqueue_nodes = [&](const unsigned long long* refined) -> int {
-    total_cap = 0;
-    for (uint32_t t = 0; t < nt; ++t) {
-      td[t].node_base = total_cap;
-      td[t].node_cap = node_cap[t];
-      total_cap += node_cap[t];
+    if (!refined) {  // not the block's first use: tile places may have changed, bounds and counters start again
+      place_nodes();
+      LOD_CK(up_.put(g_tiles, td.data(), nt * sizeof(TileDesc)));
+      LOD_CK(cudaMemsetAsync(&g_rb->nctr, 0, offsetof(NodeRead, abort) - offsetof(NodeRead, nctr), st));
     }
-    LOD_CK(up_.put(d_tiles.p, td.data(), nt * sizeof(TileDesc)));
     LOD_CK(d_nodes.alloc(total_cap * sizeof(lod_node_t)));
     LOD_CK(d_aux.alloc(total_cap * sizeof(NodeAux)));
-    LOD_CK(d_lvl.alloc(lvl.size() * 4));
-    LOD_CK(d_nn.alloc(nt * 4));
-    LOD_CK(d_leafcap.alloc(leaf_cap.size() * 8));
-    LOD_CK(d_nctr.alloc(sizeof(DevCounters)));
-    LOD_CK(cudaMemsetAsync(d_leafcap.p, 0, leaf_cap.size() * 8, st));
-    LOD_CK(cudaMemsetAsync(d_nctr.p, 0, sizeof(DevCounters), st));
     LOD_LAUNCH("nodes", 0,
-               launch_nodes(A, d_nodes.as<lod_node_t>(), d_aux.as<NodeAux>(), d_lvl.as<uint32_t>(),
-                            d_nn.as<uint32_t>(), d_leafcap.as<unsigned long long>(), d_nctr.as<DevCounters>(),
+               launch_nodes(A, d_nodes.as<lod_node_t>(), d_aux.as<NodeAux>(), g_lvl, g_nn, g_rb->leaf_cap, &g_rb->nctr,
                             refined, st));
-    LOD_CK(cudaMemcpyAsync(n_nodes.data(), d_nn.p, nt * 4, cudaMemcpyDeviceToHost, st));
-    LOD_CK(cudaMemcpyAsync(lvl.data(), d_lvl.p, lvl.size() * 4, cudaMemcpyDeviceToHost, st));
-    LOD_CK(cudaMemcpyAsync(leaf_cap.data(), d_leafcap.p, leaf_cap.size() * 8, cudaMemcpyDeviceToHost, st));
     return LOD_OK;
   };
   bool nodes_enqueued = false;
@@ -924,32 +1044,26 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   uint64_t round_chunks = n_chunks0;
   for (uint32_t round = 0;; ++round) {
     ++S.rounds;
-    // pool for this round's grids
-    std::vector<uint64_t> offs;
-    const PoolLayout L = layout_pool(srcs, round_first, round_n, &offs);
-    pools.emplace_back(new DevBuf(st, ws));
-    DevBuf& pool = *pools.back();
-    LOD_CK(pool.alloc(L.total * 4));
-    LOD_CK(cudaMemsetAsync(pool.p, 0, L.zero * 4, st));
-    uint32_t* pb = pool.as<uint32_t>();
-    A.cnt_base = pb + L.cnt;
-    A.cursor_delta = L.start - L.cnt;
-    for (uint32_t i = 0; i < round_n; ++i) {
-      SrcDesc& s = srcs[round_first + i];
-      s.ovf = pb + L.ovf + offs[4 * i + 0];
-      s.cnt = pb + L.cnt + offs[4 * i + 1];
-      s.start = pb + L.start + offs[4 * i + 2];
-      s.map = pb + L.map + offs[4 * i + 3];
+    // pool, grids and jobs of this round (the first round's are uploaded
+    // already, unless the host had to wait for the boxes)
+    const PyrJob* g_jobs = reinterpret_cast<const PyrJob*>(in + o_jobs);
+    if (round > 0 || sync_roots) {
+      const int rc = prepare_round(round_first, round_n);
+      if (rc != LOD_OK) return rc;
+      LOD_CK(up_.put(g_srcs + round_first, srcs.data() + round_first, round_n * sizeof(SrcDesc)));
+      LOD_CK(d_jobs.alloc(std::max<size_t>(jobs.size(), 1) * sizeof(PyrJob)));
+      LOD_CK(up_.put(d_jobs.p, jobs.data(), jobs.size() * sizeof(PyrJob)));
+      g_jobs = d_jobs.as<PyrJob>();
     }
-    LOD_CK(up_.put(d_srcs.as<SrcDesc>() + round_first, srcs.data() + round_first,
-                           round_n * sizeof(SrcDesc)));
+    LOD_CK(cudaMemsetAsync(pools.back()->p, 0, L.zero * 4, st));
     if (round == 0 && !sync_roots)
-      LOD_LAUNCH("roots", 0,
-                 launch_roots(d_tiles.as<TileDesc>(), d_bbox.as<int>(), d_srcs.as<SrcDesc>(), nt, T,
-                              prm.max_depth, d_abort.as<unsigned int>(), st));
-    LOD_CK(up_.put(d_nchunks.p, &round_chunks, sizeof(round_chunks)));
-    A.tiles = d_tiles.as<TileDesc>();
-    A.srcs = d_srcs.as<SrcDesc>();
+      LOD_LAUNCH("roots", 0, launch_roots(g_tiles, g_bbox, g_srcs, nt, T, prm.max_depth, &g_rb->abort, st));
+    if (round > 0) {
+      LOD_CK(up_.put(g_nchunks, &round_chunks, sizeof(round_chunks)));
+      LOD_CK(cudaMemsetAsync(&g_rb->ctr, 0, sizeof(DevCounters), st));
+    }
+    A.tiles = g_tiles;
+    A.srcs = g_srcs;
     A.tmp[0] = d_tmp0.as<int4>();
     A.tmp[1] = d_tmp1.as<int4>();
     A.tmp_idx[0] = d_tmpi0.as<uint32_t>();
@@ -959,56 +1073,31 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     uint64_t round_points = 0;
     for (uint32_t i = 0; i < round_n; ++i) round_points += srcs[round_first + i].n;
     LOD_LAUNCH("count", 16.0 * round_points,
-               launch_count(A, d_chunk_src.as<uint32_t>(), d_nchunks.as<unsigned long long>(), cgrid, st));
+               launch_count(A, g_chunk_src, g_nchunks, cgrid, st));
 
-    // pyramid jobs: up passes (bottom levels d, d-4, ...), down passes (tops 0, 4, ...)
-    std::vector<std::vector<PyrJob>> up, down;
-    for (uint32_t i = 0; i < round_n; ++i) {
-      const uint32_t sid = round_first + i;
-      const uint32_t d = srcs[sid].d;
-      uint32_t pass = 0;
-      for (int jb = (int)d; jb > 0; jb -= 4, ++pass) {
-        if (up.size() <= pass) up.emplace_back();
-        const uint32_t k = std::min<uint32_t>(4, jb);
-        const uint64_t blocks = ipow8(jb - k);
-        for (uint64_t b = 0; b < blocks; ++b) up[pass].push_back({sid, (uint32_t)jb, (uint32_t)b});
-      }
-      pass = 0;
-      for (uint32_t jt = 0; jt < d || (d == 0 && jt == 0); jt += 4, ++pass) {
-        if (down.size() <= pass) down.emplace_back();
-        const uint64_t blocks = ipow8(jt);
-        for (uint64_t b = 0; b < blocks; ++b) down[pass].push_back({sid, jt, (uint32_t)b});
-        if (d == 0) break;
-      }
-    }
-    size_t n_jobs = 0;
-    for (auto& v : up) n_jobs += v.size();
-    for (auto& v : down) n_jobs += v.size();
-    std::vector<PyrJob> all;
-    all.reserve(n_jobs);
-    for (auto& v : up) all.insert(all.end(), v.begin(), v.end());
-    for (auto& v : down) all.insert(all.end(), v.begin(), v.end());
-    LOD_CK(d_jobs.alloc(std::max<size_t>(all.size(), 1) * sizeof(PyrJob)));
-    LOD_CK(up_.put(d_jobs.p, all.data(), all.size() * sizeof(PyrJob)));
     size_t jo = 0;
-    for (auto& v : up) {
-      LOD_LAUNCH("pyramid_up", 0, launch_pyr_up(A, d_jobs.as<PyrJob>() + jo, (uint32_t)v.size(), st));
-      jo += v.size();
+    for (uint32_t n : up_jobs) {
+      LOD_LAUNCH("pyramid_up", 0, launch_pyr_up(A, g_jobs + jo, n, st));
+      jo += n;
     }
     // capacity of the source table for grids created by this round
     const uint64_t need = (uint64_t)n_src + round_points / (T + 1ull) + 16;
     if (need > src_cap) {
-      LOD_CK(d_srcs.grow(need * sizeof(SrcDesc), (size_t)n_src * sizeof(SrcDesc)));
+      DevBuf q(st, ws);
+      LOD_CK(q.alloc(need * sizeof(SrcDesc)));
+      LOD_CK(cudaMemcpyAsync(q.p, g_srcs, (size_t)n_src * sizeof(SrcDesc), cudaMemcpyDeviceToDevice, st));
+      std::swap(q.p, d_srcs_own.p);
+      std::swap(q.bytes, d_srcs_own.bytes);
+      std::swap(q.blk, d_srcs_own.blk);
       src_cap = need;
-      A.srcs = d_srcs.as<SrcDesc>();
+      g_srcs = d_srcs_own.as<SrcDesc>();
+      A.srcs = g_srcs;
     }
-    LOD_CK(cudaMemsetAsync(d_ctr.p, 0, sizeof(DevCounters), st));
     const uint32_t next_buf = 1 + (round & 1);
-    for (auto& v : down) {
+    for (uint32_t n : down_jobs) {
       LOD_LAUNCH("pyramid_down", 0,
-                 launch_pyr_down(A, d_jobs.as<PyrJob>() + jo, (uint32_t)v.size(), n_src,
-                                 (uint32_t)(src_cap - n_src), next_buf, d_ctr.as<DevCounters>(), st));
-      jo += v.size();
+                 launch_pyr_down(A, g_jobs + jo, n, n_src, (uint32_t)(src_cap - n_src), next_buf, &g_rb->ctr, st));
+      jo += n;
     }
     // the cells refined by this round (if any) go to a ping-pong buffer; it
     // is set up before the counters are known so that the scatter follows
@@ -1026,22 +1115,20 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       A.tmp_idx[1] = d_tmpi1.as<uint32_t>();
     }
     LOD_LAUNCH("scatter", 32.0 * round_points,
-               launch_scatter(A, d_chunk_src.as<uint32_t>(), d_nchunks.as<unsigned long long>(), round, cgrid, st));
+               launch_scatter(A, g_chunk_src, g_nchunks, round, cgrid, st));
     if (round == 0) {
-      const int rc = enqueue_nodes(&d_ctr.as<DevCounters>()->new_srcs);
+      const int rc = enqueue_nodes(&g_rb->ctr.new_srcs);
       if (rc != LOD_OK) return rc;
       nodes_enqueued = true;
     }
-    DevCounters* hc = static_cast<DevCounters*>(tl_stage.get(sizeof(DevCounters) + sizeof(unsigned int)));
-    if (!hc) return LOD_ERR_OOM;
-    unsigned int* h_abort = reinterpret_cast<unsigned int*>(hc + 1);
-    *h_abort = 0;
-    LOD_CK(cudaMemcpyAsync(hc, d_ctr.p, sizeof(DevCounters), cudaMemcpyDeviceToHost, st));
-    if (round == 0 && !sync_roots)
-      LOD_CK(cudaMemcpyAsync(h_abort, d_abort.p, sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-    LOD_CK(cudaStreamSynchronize(st));
+    const NodeRead* hr = nullptr;
+    {
+      const int rc = read_back(round == 0 ? rb_bytes : sizeof(DevCounters), &hr);
+      if (rc != LOD_OK) return rc;
+    }
+    const DevCounters* hc = &hr->ctr;
     clk.tick("round");
-    if (*h_abort) {
+    if (round == 0 && !sync_roots && hr->abort) {
       prof.resolve();
       return kRetryWithRoots;
     }
@@ -1063,8 +1150,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
 
     // next round: the new grids, their chunk space
     srcs.resize(n_src + new_srcs);
-    LOD_CK(cudaMemcpyAsync(srcs.data() + n_src, d_srcs.as<SrcDesc>() + n_src, new_srcs * sizeof(SrcDesc),
-                           cudaMemcpyDeviceToHost, st));
+    LOD_CK(cudaMemcpyAsync(srcs.data() + n_src, g_srcs + n_src, new_srcs * sizeof(SrcDesc), cudaMemcpyDeviceToHost, st));
     LOD_CK(cudaStreamSynchronize(st));
     clk.tick("new_srcs");
     ++S.host_syncs;
@@ -1086,15 +1172,17 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     (void)new_points;
     LOD_CK(d_chunk_src.alloc(std::max<uint64_t>(round_chunks, 1) * 4));
     LOD_CK(up_.put(d_chunk_src.p, cs.data(), round_chunks * 4));
+    g_chunk_src = d_chunk_src.as<uint32_t>();
   }
 
   // ---- node tables: check the table enqueued with the first round (or
   // build it now), growing the capacity of tiles that overflowed
   for (int attempt = 0;; ++attempt) {
     if (!nodes_enqueued) {
-      const int rc = enqueue_nodes(nullptr);
+      int rc = enqueue_nodes(nullptr);
       if (rc != LOD_OK) return rc;
-      LOD_CK(cudaStreamSynchronize(st));
+      const NodeRead* hr = nullptr;
+      if ((rc = read_back(rb_bytes, &hr)) != LOD_OK) return rc;
       clk.tick("nodes");
       up_.recycle();
       prof.resolve();
@@ -1132,8 +1220,8 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   // array starts at an estimate; if the levels need more, the phase is run
   // once more with the exact size (every step of it is idempotent).
   DevBuf d_dense(st);  // result
-  DevBuf d_stage0(st, ws), d_stage1(st, ws), d_sum0(st, ws), d_sum1(st, ws), d_pref(st, ws), d_tvox(st, ws);
-  DevBuf d_units(st, ws), d_lctr(st, ws), d_vstate(st, ws), d_order(st, ws);
+  DevBuf d_stage0(st, ws), d_stage1(st, ws), d_sum0(st, ws), d_sum1(st, ws), d_pref(st, ws);
+  DevBuf d_units(st, ws), d_vread(st, ws), d_order(st, ws);
   const bool filt = prm.mode == LOD_FILTER;
   const int n_vlev = max_levels >= 2 ? (int)max_levels - 1 : 0;  // parent levels max_levels-2 .. 0
   const size_t pstride = 2 * (size_t)(nt + 1);
@@ -1176,10 +1264,14 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   const uint32_t units_cap = (uint32_t)std::min<uint64_t>((uint64_t)max_items * 64, 1u << 20);
   LOD_CK(d_units.alloc((size_t)units_cap * sizeof(uint4)));
   LOD_CK(d_order.alloc((size_t)max_items * 4));
-  const size_t lctr_bytes = (size_t)std::max(n_vlev, 1) * sizeof(DevCounters);
-  LOD_CK(d_lctr.alloc(lctr_bytes));
-  LOD_CK(d_vstate.alloc(2 * sizeof(unsigned long long)));
-  LOD_CK(d_tvox.alloc(nt * 8));
+  // what the host reads after the levels, one block: voxels done and the
+  // array-too-small flag, every level's counters, every tile's voxels
+  const size_t vr_ctr = 2 * sizeof(unsigned long long), vr_tvox = vr_ctr + (size_t)std::max(n_vlev, 1) * sizeof(DevCounters),
+               vr_bytes = vr_tvox + nt * 8;
+  LOD_CK(d_vread.alloc(vr_bytes));
+  unsigned long long* const g_vstate = d_vread.as<unsigned long long>();
+  DevCounters* const g_lctr = reinterpret_cast<DevCounters*>(d_vread.as<char>() + vr_ctr);
+  unsigned long long* const g_tvox = reinterpret_cast<unsigned long long*>(d_vread.as<char>() + vr_tvox);
   uint64_t dense_cap = std::max<uint64_t>(M / 2, 4096);
   std::vector<DevCounters> lctr(std::max(n_vlev, 1));
   unsigned long long vstate[2] = {0, 0};
@@ -1192,14 +1284,11 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       "voxelize_L18", "voxelize_L19", "voxelize_L20", "voxelize_L21", "voxelize_L22", "voxelize_L23",
       "voxelize_L24", "voxelize_L25", "voxelize_L26", "voxelize_L27", "voxelize_L28", "voxelize_L29",
       "voxelize_L30", "voxelize_L31", "voxelize_L32", "voxelize_L33"};
-  A.tiles = d_tiles.as<TileDesc>();
   DevBuf d_rsums(st);  // result (out-of-core merges): exact sums of the roots' voxels
   for (int attempt = 0;; ++attempt) {
     LOD_CK(d_dense.alloc(dense_cap * 16));
     if (opt.keep_root_sums && filt) LOD_CK(d_rsums.alloc(dense_cap * 16));
-    LOD_CK(cudaMemsetAsync(d_tvox.p, 0, nt * 8, st));
-    LOD_CK(cudaMemsetAsync(d_lctr.p, 0, lctr_bytes, st));
-    LOD_CK(cudaMemsetAsync(d_vstate.p, 0, 2 * sizeof(unsigned long long), st));
+    LOD_CK(cudaMemsetAsync(d_vread.p, 0, vr_bytes, st));
     // optionally, every level's launches go into one CUDA graph (the
     // levels need no host round trip, so they can be captured as a unit)
     GraphCapture cap(st);
@@ -1214,12 +1303,12 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     for (int l = n_vlev - 1; l >= 0; --l) {
       const uint32_t* ip = &pref[(size_t)l * pstride];
       const uint32_t n_items = ip[nt], n_par = ip[nt + 1 + nt];
-      DevCounters* lc = d_lctr.as<DevCounters>() + l;
+      DevCounters* lc = g_lctr + l;
       const int par = (l + 1) & 1;
       vl.level = (uint32_t)l;
       vl.n_items = n_items;
       vl.item_prefix = d_pref.as<uint32_t>() + (size_t)l * pstride;
-      vl.lvl_start = d_lvl.as<uint32_t>();
+      vl.lvl_start = g_lvl;
       vl.nodes = d_nodes.as<lod_node_t>();
       vl.aux = d_aux.as<NodeAux>();
       vl.stage_out = (par ? d_stage1 : d_stage0).as<int4>();
@@ -1232,7 +1321,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       vl.units = d_units.as<uint4>();
       vl.unit_cap = units_cap;
       vl.dense_cap = dense_cap;
-      vl.vstate = d_vstate.as<unsigned long long>();
+      vl.vstate = g_vstate;
       vl.parent_prefix = d_pref.as<uint32_t>() + (size_t)l * pstride + (nt + 1);
       vl.n_parents = n_par;
       // the deepest level takes its items in node order; every level scan
@@ -1252,7 +1341,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       vox_rec[l] = prof.recs.size();
       LOD_LAUNCH("level_scan", 0,
                  launch_level_scan(A, vl, d_pref.as<uint32_t>() + (size_t)l * pstride + (nt + 1), n_par,
-                                   d_tvox.as<unsigned long long>(), lc, vst));
+                                   g_tvox, lc, vst));
     }
     if (n_vlev > 0) {
       // the roots' voxels: the items of the top level have no parent pass
@@ -1262,10 +1351,13 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       vl.root_sums = nullptr;
     }
     if (use_graph) LOD_CK(cap.launch());
-    LOD_CK(cudaMemcpyAsync(lctr.data(), d_lctr.p, lctr_bytes, cudaMemcpyDeviceToHost, st));
-    LOD_CK(cudaMemcpyAsync(vstate, d_vstate.p, sizeof(vstate), cudaMemcpyDeviceToHost, st));
-    LOD_CK(cudaMemcpyAsync(tvox.data(), d_tvox.p, nt * 8, cudaMemcpyDeviceToHost, st));
+    char* const hv = static_cast<char*>(tl_stage.get(vr_bytes));
+    if (!hv) return LOD_ERR_OOM;
+    LOD_CK(cudaMemcpyAsync(hv, d_vread.p, vr_bytes, cudaMemcpyDeviceToHost, st));
     LOD_CK(cudaStreamSynchronize(st));
+    std::memcpy(vstate, hv, sizeof(vstate));
+    std::memcpy(lctr.data(), hv + vr_ctr, lctr.size() * sizeof(DevCounters));
+    std::memcpy(tvox.data(), hv + vr_tvox, nt * 8);
     clk.tick("voxels");
     ++S.host_syncs;
     for (int l = 0; l < n_vlev; ++l)
@@ -1333,7 +1425,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     for (uint32_t t = 0; t < nt; ++t) max_nodes = std::max(max_nodes, n_nodes[t]);
     LOD_CK(d_vpts.alloc(dense_cap * 16));
     LOD_LAUNCH("voxel_points", 32.0 * V,
-               launch_voxel_points(d_tiles.as<TileDesc>(), nt, d_nodes.as<lod_node_t>(), d_nn.as<uint32_t>(), max_nodes,
+               launch_voxel_points(g_tiles, nt, d_nodes.as<lod_node_t>(), g_nn, max_nodes,
                                    d_dense.as<int4>(), d_vpts.as<int4>(), st));
   }
   up_.recycle();
