@@ -598,9 +598,16 @@ __device__ __forceinline__ unsigned long long* pick_keys() { return reinterpret_
 __device__ __forceinline__ uint2* pick_pays() { return reinterpret_cast<uint2*>(vox_fields()) + kCapPick; }
 __device__ __forceinline__ uint32_t* pick_counts() { return vox_fields() + 4u * kCapPick; }
 
+// The upper word of a sample's key (first come: the key is the 32-bit index
+// itself, unique, so it takes the upper word's place).
+template <int MODE>
+__device__ __forceinline__ uint32_t pick_high(uint32_t ix, uint32_t level) {
+  return MODE == LOD_FIRST ? ix : (uint32_t)(pick_key<MODE>(ix, level) >> 32);
+}
+
 template <int MODE>
 __device__ __forceinline__ void pick_sample(const PickArgs& P, uint32_t rk, uint32_t cell, uint32_t ix, uint32_t rgba, uint32_t n) {
-  const uint32_t h = (uint32_t)(pick_key<MODE>(ix, P.level) >> 32);
+  const uint32_t h = pick_high<MODE>(ix, P.level);
   const unsigned long long mine = ((unsigned long long)h << 32) | ix;
   const unsigned long long old = atomicMin(&pick_keys()[rk], mine);
   if (atomicAdd(&pick_counts()[rk], n) == 0u) vox_cells<5, kCapPick>()[rk] = (uint16_t)cell;
@@ -913,7 +920,7 @@ __device__ __forceinline__ void extract_pick(const PickArgs& P) {
     pick_keys()[i] = ~0ull;
     pick_counts()[i] = 0u;
     if (pay.x != best) S.settle = 1u;
-    else if (best >= P.idx_bound || (uint32_t)(pick_key<MODE>(best, P.level) >> 32) != (uint32_t)(e >> 32))
+    else if (best >= P.idx_bound || pick_high<MODE>(best, P.level) != (uint32_t)(e >> 32))
       atomicOr(P.error, kErrInternal);  // cannot happen for a cell that received a sample
     if (P.out_at + i < P.stage_cap)
       P.stage_out[P.out_at + i] = make_int4((int)parent_cell(cell, S.I), (int)pay.y, (int)n, (int)best);
