@@ -909,6 +909,7 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
         // contribute to its parent (all nodes), and the exact leaf points
         atomicAdd(&leaf_cap[lvl], (unsigned long long)umin64(cnt, kOctCells));
         if (!split) atomicAdd(&leaf_cap[kMaxLevels + 1 + lvl], (unsigned long long)cnt);
+        else atomicAdd(&leaf_cap[2 * (kMaxLevels + 1)], (unsigned long long)umin64(cnt, kVoxelGuess));
         if (split) {
           const uint32_t half = lg - 1;
           uint32_t r = 0;
