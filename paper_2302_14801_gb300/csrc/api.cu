@@ -224,21 +224,24 @@ int lod_render(const lod_result_t* r, const lod_camera_t* cam, uint64_t* d_frame
   const uint64_t pixels = (uint64_t)c.width * c.height;
   cudaError_t e = cudaMemsetAsync(d_framebuffer, 0xFF, pixels * 8, st);
   if (e != cudaSuccess) return to_status(e);
-  // scratch: drawn-node flags and two counters
+  // scratch: three counters, the draw list and drawn-node flags
   void* scratch = nullptr;
-  const size_t cnt_off = ((size_t)v.n_nodes + 15) & ~size_t(15);
-  e = cudaMallocAsync(&scratch, cnt_off + 16, st);
+  const size_t list_bytes = lodk::render_list_entries(v.n_nodes, v.n_points, v.n_voxels) * sizeof(uint2);
+  e = cudaMallocAsync(&scratch, 16 + list_bytes + v.n_nodes, st);
   if (e != cudaSuccess) return to_status(e);
-  unsigned long long* drawn = reinterpret_cast<unsigned long long*>(static_cast<char*>(scratch) + cnt_off);
+  unsigned long long* drawn = static_cast<unsigned long long*>(scratch);
   unsigned int* n_vis = reinterpret_cast<unsigned int*>(drawn + 1);
+  unsigned int* n_list = n_vis + 1;
+  uint2* list = reinterpret_cast<uint2*>(static_cast<char*>(scratch) + 16);
+  uint8_t* visible = static_cast<uint8_t*>(scratch) + 16 + list_bytes;
   e = cudaMemsetAsync(drawn, 0, 16, st);
   int dev = 0, sms = 1;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
     e = lodk::launch_render(v.nodes, v.n_nodes, reinterpret_cast<const int4*>(v.points),
-                            reinterpret_cast<const int4*>(v.voxels), c, static_cast<uint8_t*>(scratch), n_vis,
-                            reinterpret_cast<unsigned long long*>(d_framebuffer), drawn, sms, st);
+                            reinterpret_cast<const int4*>(v.voxels), c, visible, n_vis, list, n_list,
+                            reinterpret_cast<unsigned long long*>(d_framebuffer), stats ? drawn : nullptr, sms, st);
   unsigned long long host[2] = {0, 0};
   if (e == cudaSuccess && stats) {
     e = cudaMemcpyAsync(host, drawn, 16, cudaMemcpyDeviceToHost, st);
@@ -249,7 +252,7 @@ int lod_render(const lod_result_t* r, const lod_camera_t* cam, uint64_t* d_frame
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
     stats->samples_drawn = host[0];
-    stats->visible_nodes = (uint32_t)host[1];
+    stats->visible_nodes = (uint32_t)host[1];  // the low half: the draw list's length lies above it
   }
   return LOD_OK;
 }

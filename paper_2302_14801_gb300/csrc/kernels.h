@@ -130,8 +130,11 @@ cudaError_t launch_merge(uint32_t mode, const MergeJob* jobs, uint32_t n_jobs, c
                          const MergeOut& o, int ctas, cudaStream_t st);
 
 // ----- rendering (Section 5) -----
+// Entries that the draw list of a frame needs room for.
+uint64_t render_list_entries(uint32_t n_nodes, uint64_t n_points, uint64_t n_voxels);
+// drawn: receives the number of samples drawn, or null.
 cudaError_t launch_render(const lod_node_t* nodes, uint32_t n_nodes, const int4* points, const int4* voxels,
-                          const lod_camera_t& cam, uint8_t* visible, unsigned int* n_visible,
-                          unsigned long long* fb, unsigned long long* drawn, int sms, cudaStream_t st);
+                          const lod_camera_t& cam, uint8_t* visible, unsigned int* n_visible, uint2* list,
+                          unsigned int* n_list, unsigned long long* fb, unsigned long long* drawn, int sms, cudaStream_t st);
 
 }  // namespace lodk
