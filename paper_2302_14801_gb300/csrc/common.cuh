@@ -52,9 +52,10 @@ struct TileDesc {
 // (Section 4.1.5).  Its points occupy [pt_off, pt_off + n) of the tile.
 struct SrcDesc {
   uint32_t* cnt;       // count pyramid, levels 0..d (level j: 8^j cells)
-  uint32_t* start;     // start pyramid (tile-relative positions); its
-                       // bottom level is the scatter cursor
-  uint32_t* map;       // bottom cells: child source id where overflowing
+  uint32_t* start;     // start pyramid (tile-relative positions); the entries of
+                       // leaves and of refined cells are the scatter's cursors
+  uint32_t* map;       // bottom cells: child source id where overflowing, else (occupied
+                       // cells) the cursor of the cell's leaf, an index into the start region
   uint32_t* ovf;       // bottom cells: overflow bit mask
   int32_t min[3];
   uint32_t tile;

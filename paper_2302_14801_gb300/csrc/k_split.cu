@@ -10,9 +10,9 @@
 // to 256^3 cells, deep refinement grids) count through a per-CTA
 // shared-memory hash table of the cells the CTA's chunks touch.  Every
 // counted cell is published with one global atomic and listed as (cell,
-// count), so that the scatter claims one block of positions per listed
-// cell; cells that miss the table or the list use warp-aggregated global
-// atomics on their cursor.  Grid pyramids (per-level sums and
+// count), so that the scatter claims one block of positions per leaf of its
+// listed cells; cells that miss the table or the list use global atomics on
+// their leaf's cursor.  Grid pyramids (per-level sums and
 // exclusive-scan starts) are built in 4-level blocks in shared memory.
 // With kept input indices the scatter writes one full 32-byte sector per
 // point.  The root cubes are computed on the device (no host round trip
@@ -510,6 +510,7 @@ __global__ void __launch_bounds__(512) k_pyr_down(BuildArgs a, const PyrJob* __r
   if (a.abort && *a.abort) return;
   __shared__ uint32_t cnt[8 + 64 + 512 + 4096];
   __shared__ uint32_t sta[1 + 8 + 64 + 512 + 4096];
+  __shared__ uint32_t s_leaf;
   const PyrJob job = jobs[blockIdx.x];
   const uint32_t sid = job.src;
   const SrcDesc s = a.srcs[sid];
@@ -537,8 +538,23 @@ __global__ void __launch_bounds__(512) k_pyr_down(BuildArgs a, const PyrJob* __r
     }
     sta[0] = top;
   }
+  uint32_t* const start_base = a.cnt_base + a.cursor_delta;
+  if (k == 0) {  // a one-cell grid (d == 0) never overflows: its start is set above
+    if (threadIdx.x == 0) s.map[0] = (uint32_t)(s.start - start_base);
+    return;
+  }
+  // the leaf that holds the whole block, if one does: the highest of the
+  // block's ancestors and itself with at most T points
+  if (threadIdx.x < 32) {
+    const uint32_t j = threadIdx.x;
+    const bool fits = j <= jt && s.cnt[pyr_off(j) + (job.block >> (3u * (jt - min(j, jt))))] <= a.T;
+    const unsigned any = __ballot_sync(0xFFFFFFFFu, fits);
+    if (j == 0) {
+      const uint32_t l = any ? (uint32_t)__ffs(any) - 1u : 0u;
+      s_leaf = any ? (uint32_t)(s.start + pyr_off(l) + (job.block >> (3u * (jt - l))) - start_base) : kNone;
+    }
+  }
   __syncthreads();
-  if (k == 0) return;  // a one-cell grid (d == 0) never overflows: its start is set above
   // sta layout: level 0 at [0], level i at 1 + lo[i]
   for (uint32_t i = 1; i <= k; ++i) {
     const uint32_t n_par = lsz[i - 1];
@@ -556,11 +572,23 @@ __global__ void __launch_bounds__(512) k_pyr_down(BuildArgs a, const PyrJob* __r
     __syncthreads();
   }
   if (jt + k != s.d) return;
-  // bottom level of the source: detect cells to refine
+  // bottom level of the source: every occupied cell's leaf, for the scatter
+  // (the highest cell above it with at most T points, or itself)
+  const uint32_t nbot = lsz[k];
+  for (uint32_t q = threadIdx.x; q < nbot; q += blockDim.x) {
+    if (!cnt[lo[k] + q]) continue;
+    uint32_t m = s_leaf;
+    if (m == kNone) {
+      uint32_t i = 1;
+      while (i < k && cnt[lo[i] + (q >> (3u * (k - i)))] > a.T) ++i;
+      m = (uint32_t)(s.start + pyr_off(jt + i) + (uint64_t)job.block * lsz[i] + (q >> (3u * (k - i))) - start_base);
+    }
+    s.map[job.block * nbot + q] = m;
+  }
+  // detect cells to refine (their map entry becomes the child grid)
   const uint32_t level_b = s.level + s.d;
   const uint32_t log2_b = s.log2size - s.d;
   if (!(level_b < a.max_depth && log2_b > 0)) return;
-  const uint32_t nbot = lsz[k];
   for (uint32_t q = threadIdx.x; q < nbot; q += blockDim.x) {
     const uint32_t n = cnt[lo[k] + q];
     if (n <= a.T) continue;
@@ -603,14 +631,40 @@ cudaError_t launch_pyr_down(const BuildArgs& a, const PyrJob* jobs, uint32_t n_j
 }
 
 // ------------------------------------------------------------------- scatter
-// Section 4.1.4 (insert): every point goes to its cell's cursor; points of
-// cells that will be refined go to the ping-pong buffer of the next round,
-// all others to their final place in the leaf-point array.  For large grids
-// the CTA re-creates its counting table from its list, claims one block of
-// positions per cell with one global atomic, and hands out positions inside
-// the block with shared-memory atomics (the CTA processes the same chunks as
-// in the counting pass).  Dense small grids claim cursors per point (one
-// atomic per warp when all its points share a cell).
+// Section 4.1.4 (insert): every point goes to the cursor of its leaf, the
+// highest cell above it with at most T points (a run of the leaf-point array;
+// the order inside a leaf is free); points of cells that will be refined go
+// to the ping-pong buffer of the next round, at their cell's cursor.  The CTA
+// re-creates its counting table from its list (it processes the same chunks
+// as in the counting pass), claims one block of positions per leaf with one
+// global atomic, and hands out positions inside the block with shared-memory
+// atomics.
+//
+// What bounds it: the random writes.  Every CTA keeps one partly written line
+// open per block, and a line that leaves L2 before it is full costs memory
+// a read and two writes.  One block per leaf instead of one per grid cell (a
+// leaf spans several cells of the grid, which is a level or two deeper than
+// most leaves) keeps a half to a quarter as many lines open: 50M aerial
+// points in random order 1.02 -> 0.84 ms, 500M indoor points (all rounds) 5.78 ->
+// 5.19 ms, 48 tiles 0.22 -> 0.16 ms.
+// (Claiming small batches from shared cursors instead, so that all CTAs fill
+// the same lines, brought the traffic down to the points themselves but needs
+// 0.8 global atomics a point: 17 % slower on 50M aerial points, 40 % on 500M
+// indoor points.)
+
+namespace {
+
+constexpr uint32_t kLeafSlots = 8192;  // table of a CTA's leaves (the rest of its shared memory)
+// keys, then the cells' leaf slots (bit 15: the cell is refined), then leaf keys and cursors
+constexpr uint32_t kScatSmem = kPrivSlots * 6u + kLeafSlots * 8u;
+
+// Where a cell's points take their places: the cursor of its leaf, or its own
+// when it is refined (an index into the start region).
+__device__ __forceinline__ uint32_t leaf_cursor(const BuildArgs& a, const SrcDesc& s, uint32_t cell, bool refined) {
+  return refined ? (uint32_t)(s.start + pyr_off(s.d) + cell - (a.cnt_base + a.cursor_delta)) : s.map[cell];
+}
+
+}  // namespace
 
 __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t* __restrict__ chunk_src,
                                                     const unsigned long long* __restrict__ n_chunks_p,
@@ -618,11 +672,11 @@ __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t*
   if (a.abort && *a.abort) return;
   __shared__ SrcDesc s;
   __shared__ uint32_t s_ovf[kSmemBins / 32];  // overflow mask of a dense grid
-  // kPrivSlots keys, kPrivSlots cursors, kPrivSlots overflow flags
   extern __shared__ __align__(16) uint32_t ptab[];
   uint32_t* pkeys = ptab;
-  uint32_t* pcur = ptab + kPrivSlots;
-  uint8_t* pflag = reinterpret_cast<uint8_t*>(ptab + 2 * kPrivSlots);
+  uint16_t* pleaf = reinterpret_cast<uint16_t*>(ptab + kPrivSlots);
+  uint32_t* lkeys = ptab + kPrivSlots + kPrivSlots / 2;
+  uint32_t* lcur = lkeys + kLeafSlots;
   const uint64_t n_chunks = *n_chunks_p;
   const uint64_t per = (n_chunks + gridDim.x - 1) / gridDim.x;
   const uint64_t c0 = (uint64_t)blockIdx.x * per;
@@ -630,32 +684,19 @@ __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t*
   int4* ovf_dst = (round & 1) ? a.tmp[1] : a.tmp[0];
   uint32_t* ovf_idx = (round & 1) ? a.tmp_idx[1] : a.tmp_idx[0];
   const uint32_t lane = lane_id();
-  // claim this CTA's block of every cell it counted
+  // claim this CTA's block of every leaf it counted points of
   for (uint32_t i = threadIdx.x; i < kPrivSlots; i += blockDim.x) pkeys[i] = 0u;
+  for (uint32_t i = threadIdx.x; i < kLeafSlots; i += blockDim.x) lkeys[i] = lcur[i] = 0u;
   __syncthreads();
+  uint32_t* const start_base = a.cnt_base + a.cursor_delta;
   {
     const uint32_t len = a.list_len[blockIdx.x];
     const uint2* list = a.lists + (uint64_t)blockIdx.x * kPrivSlots;
     // the listed cells belong to the CTA's sources, whose count regions are
-    // laid out in source order: a binary search finds each cell's source,
-    // whose overflow bit is kept beside the cursor
+    // laid out in source order: a binary search finds each cell's source
     const uint32_t sid_lo = c0 < c1 ? chunk_src[c0] : 0u, sid_hi = c0 < c1 ? chunk_src[c1 - 1] : 0u;
     for (uint32_t j = threadIdx.x; j < len; j += blockDim.x) {
       const uint2 e = list[j];
-      // bounded probing, as in the counting pass: a cell that does not find
-      // a slot near its home claims nothing here, and its points take
-      // positions from the cell's global cursor instead
-      uint32_t slot = priv_home(e.x + 1u);
-      bool placed = false;
-      for (uint32_t probe = 0; probe < kPrivProbe; ++probe) {
-        if (atomicCAS(&pkeys[slot], 0u, e.x + 1u) == 0u) {
-          placed = true;
-          break;
-        }
-        slot = (slot + 1 == kPrivSlots) ? 0u : slot + 1;
-      }
-      if (!placed) continue;
-      pcur[slot] = atomicAdd(a.cnt_base + e.x + a.cursor_delta, e.y);
       uint32_t lo = sid_lo, hi = sid_hi;  // last source whose count region starts at or before e.x
       while (lo < hi) {
         const uint32_t mid = (lo + hi + 1) >> 1;
@@ -664,8 +705,50 @@ __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t*
       }
       const SrcDesc& es = a.srcs[lo];
       const uint32_t cell = e.x - (uint32_t)(es.cnt + pyr_off(es.d) - a.cnt_base);
-      pflag[slot] = (uint8_t)((es.ovf[cell >> 5] >> (cell & 31u)) & 1u);
+      const uint32_t refined = (es.ovf[cell >> 5] >> (cell & 31u)) & 1u;
+      const uint32_t leaf1 = leaf_cursor(a, es, cell, refined != 0u) + 1u;
+      // bounded probing in both tables, as in the counting pass: a cell that
+      // does not find a slot near its home (or whose leaf does not) claims
+      // nothing here, and its points take positions from the leaf's global
+      // cursor instead.  The leaf's slot comes first: a cell is only entered
+      // with it.
+      uint32_t l = __umulhi(leaf1 * 0x9E3779B1u, kLeafSlots);
+      bool placed = false;
+      for (uint32_t probe = 0; probe < kPrivProbe; ++probe) {
+        const uint32_t old = atomicCAS(&lkeys[l], 0u, leaf1);
+        if (old == 0u || old == leaf1) {
+          placed = true;
+          break;
+        }
+        l = (l + 1 == kLeafSlots) ? 0u : l + 1;
+      }
+      if (!placed) continue;
+      uint32_t slot = priv_home(e.x + 1u);
+      placed = false;
+      for (uint32_t probe = 0; probe < kPrivProbe; ++probe) {
+        if (atomicCAS(&pkeys[slot], 0u, e.x + 1u) == 0u) {
+          placed = true;
+          break;
+        }
+        slot = (slot + 1 == kPrivSlots) ? 0u : slot + 1;
+      }
+      if (!placed) continue;
+      pleaf[slot] = (uint16_t)(l | (refined << 15));
+      atomicAdd(&lcur[l], e.y);
     }
+  }
+  __syncthreads();
+  {  // all claims of a thread in flight together
+    constexpr int kMine = (int)(kLeafSlots / kBlock);
+    uint32_t k1[kMine], at[kMine];
+#pragma unroll
+    for (int i = 0; i < kMine; ++i) {
+      k1[i] = lkeys[threadIdx.x + i * kBlock];
+      if (k1[i]) at[i] = atomicAdd(start_base + k1[i] - 1u, lcur[threadIdx.x + i * kBlock]);
+    }
+#pragma unroll
+    for (int i = 0; i < kMine; ++i)
+      if (k1[i]) lcur[threadIdx.x + i * kBlock] = at[i];
   }
   __syncthreads();
   uint32_t cur = kNone;
@@ -688,7 +771,6 @@ __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t*
         s.buf == 0 ? td.in_idx : (s.buf == 1 ? a.tmp_idx[0] : a.tmp_idx[1]) + td.pt_base + s.pt_off;
     const uint64_t first = (c - s.chunk0) << kChunkLog2;
     const uint64_t end = min(first + kChunk, (uint64_t)s.n);
-    uint32_t* cursor = s.start + pyr_off(s.d);
     const int32_t mx = s.min[0], my = s.min[1], mz = s.min[2];
     const uint32_t lg = s.log2size, d = s.d;
     const bool priv = s.priv != 0;
@@ -714,21 +796,26 @@ __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t*
       pb[k] = 0;
       if (!v) continue;
       const uint32_t bin = bins[k];
-      // the CTA's block of the cell (claimed from its list), else the
-      // cell's global cursor (cells the list had no room for)
+      // the CTA's block of the leaf (claimed from its list), else the leaf's
+      // global cursor (cells and leaves the tables had no room for)
       const int slot = priv_find(pkeys, kbase + bin + 1u);
-      const int leader = __ffs(m) - 1;
-      const int s0 = __shfl_sync(m, slot, leader);
-      const uint32_t b0 = __shfl_sync(m, bin, leader);
-      if (__all_sync(m, slot == s0 && bin == b0)) {
-        agg |= 1u << k;  // the whole warp's points share one cell: one claim
-        if ((int)lane == leader)
-          pb[k] = s0 >= 0 ? atomicAdd(&pcur[s0], (uint32_t)__popc(m)) : atomicAdd(cursor + bin, (uint32_t)__popc(m));
+      uint32_t f, l = kNone;
+      if (slot >= 0) {
+        const uint32_t e = pleaf[slot];
+        f = e >> 15;
+        l = e & 0x7FFFu;
       } else {
-        pb[k] = slot >= 0 ? atomicAdd(&pcur[slot], 1u) : atomicAdd(cursor + bin, 1u);
+        const uint32_t* om = priv ? s.ovf : s_ovf;
+        f = (om[bin >> 5] >> (bin & 31u)) & 1u;
       }
-      const uint32_t* om = priv ? s.ovf : s_ovf;
-      const uint32_t f = slot >= 0 ? (uint32_t)pflag[slot] : (om[bin >> 5] >> (bin & 31u)) & 1u;
+      const int leader = __ffs(m) - 1;
+      const uint32_t l0 = __shfl_sync(m, l, leader);
+      if (__all_sync(m, l == l0 && l0 != kNone)) {
+        agg |= 1u << k;  // the whole warp's points share one leaf: one claim
+        if ((int)lane == leader) pb[k] = atomicAdd(&lcur[l0], (uint32_t)__popc(m));
+      } else {
+        pb[k] = l != kNone ? atomicAdd(&lcur[l], 1u) : atomicAdd(start_base + leaf_cursor(a, s, bin, f != 0u), 1u);
+      }
       ovf_bits |= f << k;
     }
 #pragma unroll
@@ -759,11 +846,11 @@ __global__ void __launch_bounds__(kBlock) k_scatter(BuildArgs a, const uint32_t*
 cudaError_t launch_scatter(const BuildArgs& a, const uint32_t* chunk_src, const unsigned long long* n_chunks,
                            uint32_t round, int grid, cudaStream_t st) {
   static bool once = [] {
-    cudaFuncSetAttribute(k_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(9 * kPrivSlots));
+    cudaFuncSetAttribute(k_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatSmem);
     return true;
   }();
   (void)once;
-  k_scatter<<<grid, kBlock, 9 * kPrivSlots, st>>>(a, chunk_src, n_chunks, round);
+  k_scatter<<<grid, kBlock, kScatSmem, st>>>(a, chunk_src, n_chunks, round);
   note_launch();
   return cudaGetLastError();
 }
@@ -900,8 +987,8 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
       if (valid && fits) {
         const SrcDesc& sd = a.srcs[sid];
         const uint32_t st = sd.start[pyr_off(j) + c];
-        // bottom cells: the start array was advanced by the scatter (cursor)
-        nd[i].point_offset = (j < sd.d) ? st : st - (uint32_t)cnt;
+        // a leaf's start was advanced over its points by the scatter (its cursor)
+        nd[i].point_offset = split ? st : st - (uint32_t)cnt;
         nd[i].child_mask = (uint8_t)mask;
         nd[i].flags = split ? 0 : (LOD_NODE_LEAF | (cnt > a.T ? LOD_NODE_OVERFULL : 0));
         nd[i].first_child = split ? next + pos : kNone;
