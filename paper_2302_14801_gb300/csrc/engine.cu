@@ -1430,7 +1430,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     for (uint32_t t = 0; t < nt; ++t) max_nodes = std::max(max_nodes, n_nodes[t]);
     LOD_CK(d_vpts.alloc(dense_cap * 16));
     LOD_LAUNCH("voxel_points", 32.0 * V,
-               launch_voxel_points(g_tiles, nt, d_nodes.as<lod_node_t>(), g_nn, max_nodes,
+               launch_voxel_points(g_tiles, nt, d_nodes.as<lod_node_t>(), g_nn, max_nodes, V,
                                    d_dense.as<int4>(), d_vpts.as<int4>(), st));
   }
   up_.recycle();
