@@ -40,6 +40,8 @@
 // each parent one contiguous voxel range (children are consecutive in node
 // order), and the next level up copies the records to that range while it
 // reads them (so each record is read once).
+#include <cstddef>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "wgrid.cuh"
@@ -390,18 +392,18 @@ __device__ __forceinline__ uint64_t child_record(const VoxShared& S, uint32_t f,
   return S.cstage[ci] + (f - S.cpre[ci]);
 }
 
-// Pass 1 of an inner child: mark its voxels and, with `dense`, publish them
-// there (idempotent; an array found too small makes the build rerun with the
+// Pass 1 of an inner child: mark its voxels [first, total) and, with `dense`,
+// publish them there (idempotent; an array found too small makes the build rerun with the
 // exact size).  Filtered records are published without their packed sums.
 template <bool FILT>
-__device__ __forceinline__ void mark_inner(const int4* stage_in, uint32_t total, int4* dense, uint64_t dense_cap) {
+__device__ __forceinline__ void mark_inner(const int4* stage_in, uint32_t first, uint32_t total, int4* dense, uint64_t dense_cap) {
   const VoxShared& S = vox_shared();
   uint32_t cl = 0, cp = 0;  // children of the samples being loaded and marked
   auto load = [&](uint32_t f, int4& q) {
     q = make_int4(0, 0, 0, 0);
     if (f < total) q = __ldcg(stage_in + child_record(S, f, cl));
   };
-  uint32_t f = threadIdx.x;
+  uint32_t f = first + threadIdx.x;
   int4 q0, q1, q2, q3;
   load(f, q0), load(f + kVoxThreads, q1), load(f + 2 * kVoxThreads, q2), load(f + 3 * kVoxThreads, q3);
   for (; f < total; f += kBatch) {
@@ -929,26 +931,14 @@ __device__ __forceinline__ void extract_pick(const PickArgs& P) {
 
 }  // namespace
 
-// Voxelize one item (a child node c of an inner node p at level v.level):
-// all of its ranks, or, for a queued unit (r_unit, p_unit), the ranks
-// [D r / P, D (r + 1) / P) of its D occupied cells.  `first`: the item's
-// first attempt, which reserves the item's staging block (D records) and,
-// when its cells need several accumulate passes, may queue the ranges after
-// the first for the partition kernel.  The CTA that holds range 0 also
-// publishes what it reads (the leaf's points, the children's voxels).
-// `next_item` (first attempts): where thread 0 leaves the item the CTA
-// takes next, fetched while this one is marked.  `split_unit`: a range of an
-// item split up front.
-template <int MODE>
-__device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, DevCounters* __restrict__ ctr, uint32_t it,
-                                         uint32_t r_unit, uint32_t p_unit, bool first, uint32_t* next_item,
-                                         bool split_unit = false) {
+namespace {
+
+// The item's header, read by warp 0 in two dependent steps: lane 0 reads the
+// child node; then lane 8 reads the parent node while lanes 0..7 read the
+// children's records (inner items), all at once.
+__device__ __forceinline__ void vox_header(const BuildArgs& a, const VoxLevel& v, uint32_t it) {
   VoxShared& S = vox_shared();
-  uint4* const bits4 = reinterpret_cast<uint4*>(vox_smem);
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-  // The item's header, read by warp 0 in two dependent steps: lane 0 reads
-  // the child node; then lane 8 reads the parent node while lanes 0..7 read
-  // the children's records (inner items), all at once.
+  const uint32_t tid = threadIdx.x, lane = tid & 31u;
   if (tid < 32) {
     if (lane == 0) {
       const uint32_t t = find_tile(v.item_prefix, a.n_tiles, it);
@@ -1015,33 +1005,15 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       S.cpre[lane + 1] = incl;
     }
   }
-#pragma unroll
-  for (uint32_t i = 0; i < kWords / 4u / kVoxThreads; ++i) bits4[tid + i * kVoxThreads] = make_uint4(0u, 0u, 0u, 0u);
-  __syncthreads();
-  constexpr bool WEIGHTED = MODE == LOD_WEIGHTED, PICKLIKE = MODE != LOD_FILTER && !WEIGHTED;  // one sample kept per cell
-  const bool leaf = S.I.leaf;
-  const bool lead = r_unit == 0;  // the one CTA of the item that publishes the children's voxels
-  // the units of an item split up front run side by side, so each of them
-  // publishes the leaf (the same values) that its later passes read
-  const bool own_leaf = lead || split_unit;
-  const uint32_t total = leaf ? (uint32_t)S.I.n : S.cpre[S.nch];  // samples
-  // the next item's counter value; its latency hides behind the mark pass
-  uint32_t next_k = 0;
-  if (next_item && tid == 0) next_k = atomicAdd(&ctr->item_head, 1u);
+}
 
-  if (WEIGHTED && tid < (uint32_t)__popc(S.pmask)) S.border[tid] = v.border[S.pfirst + tid];
-
-  // ---- pass 1: mark the occupied cells
-  if (!leaf) mark_inner<MODE == LOD_FILTER>(v.stage_in, total, lead ? v.dense : nullptr, v.dense_cap);
-  else if (a.wide) mark_wide(a.wide + 2 * S.pbase, total, own_leaf ? a.out + S.pbase : nullptr, own_leaf ? a.out_idx + S.pbase : nullptr);
-  else mark_leaf(a.out + S.pbase, total);
-  __syncthreads();
-
-  // ---- rank the occupied cells: exclusive scan of the words' counts.  Every
-  // warp ranks 32 kScan consecutive groups of four words by coalesced 16-byte
-  // loads: lane l holds groups l, l + 32, ...
-  uint32_t next_it = next_k;
-  if (next_item && tid == 0 && v.order && next_k < v.n_items) next_it = v.order[next_k];
+// Ranks the occupied cells: an exclusive scan of the words' counts.  Every
+// warp ranks 32 kScan consecutive groups of four words by coalesced 16-byte
+// loads: lane l holds groups l, l + 32, ...  Returns their number.
+__device__ __forceinline__ uint32_t vox_rank_cells() {
+  VoxShared& S = vox_shared();
+  const uint4* const bits4 = reinterpret_cast<const uint4*>(vox_smem);
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   uint32_t D;
   {
     uint32_t pre[kScan], tot = 0;
@@ -1082,47 +1054,29 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       reinterpret_cast<uint2*>(vox_wrank())[at] = make_uint2(r0 | (r1 << 16), r2 | (r3 << 16));
     }
   }
-  // the narrowest sums that provably cannot overflow for the points of this cube
-  const SumLayout lay = leaf && S.I.npts <= kLeafMaxSamples ? kLeaf16 : (S.I.npts <= kNarrowMaxSamples ? kNarrow : kWide);
-  const uint32_t cap = PICKLIKE ? kCapPick : WEIGHTED ? kCapWeighted : (lay == kLeaf16 ? kCapLeaf : (lay == kNarrow ? kCapNarrow : kCapWide));
-  const uint32_t C = (v.range_cells && v.range_cells < cap) ? v.range_cells : cap;  // ranks per pass
-  // thread 0: the item's first staging record.  The reservation (or, for
-  // a unit, the read of the first attempt's) is issued here and its value
-  // first used before the first extraction, so its latency overlaps the
-  // accumulate pass.
-  unsigned long long stg = 0;
-  if (tid == 0) {
-    S.D = D;
-    if (first) {
-      stg = atomicAdd(v.stage_used, (unsigned long long)D);
-      v.aux[S.I.g].occ = D;
-      S.r0 = 0;
-      S.r1 = D;
-      const uint32_t P = (D + C - 1) / C;
-      if (P > 1) atomicAdd(&ctr->vox_retries, 1ull);
-      uint32_t q0 = 0;
-      if (P > 1 && v.units && P >= v.queue_ranges && reserve_units(&ctr->units, v.unit_cap, P - 1, &q0)) {
-        for (uint32_t r = 1; r < P; ++r) v.units[q0 + r - 1] = make_uint4(it, r, P, 0u);
-        S.r1 = D / P;
-      }
-    } else {
-      stg = v.aux[S.I.g].stage;  // reserved by the first attempt, or by the up-front split
-      S.r0 = (uint32_t)((uint64_t)D * r_unit / p_unit);
-      S.r1 = (uint32_t)((uint64_t)D * (r_unit + 1) / p_unit);
-      if (r_unit == 0) v.aux[S.I.g].occ = D;
-    }
-    S.n_wraps = 0;
-    S.settle = 0;
-  }
-  __syncthreads();
+  return D;
+}
 
-  // ---- pass 2: accumulate the ranks [lo, lo + span), one pass per range
-  // (a leaf read from 32-byte staging records was published by the mark pass:
-  // later passes read the 16- or 20-byte copy)
-  uint32_t passes = 1;
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// Pass 2 over the ranks [S.r0, S.r1), C of them at a time: accumulate, then
+// extract.  (A leaf read from 32-byte staging records was published by the
+// mark pass: these passes read the 16- or 20-byte copy.)  The item's first
+// staging record: thread 0 brings it in `stg`, or (CLUSTER) S.stage holds it
+// once the cluster barrier that every thread has arrived at is complete; the
+// first extraction, or the end if there is none, waits for that.
+template <int MODE, bool CLUSTER>
+__device__ __forceinline__ void vox_ranges(const BuildArgs& a, const VoxLevel& v, DevCounters* __restrict__ ctr, SumLayout lay,
+                                           uint32_t C, unsigned long long stg) {
+  VoxShared& S = vox_shared();
+  constexpr bool WEIGHTED = MODE == LOD_WEIGHTED, PICKLIKE = MODE != LOD_FILTER && !WEIGHTED;
+  const uint32_t tid = threadIdx.x;
+  const bool leaf = S.I.leaf;
+  const uint32_t total = leaf ? (uint32_t)S.I.n : S.cpre[S.nch];
+  bool waited = !CLUSTER;
   for (uint32_t lo = S.r0, r1 = S.r1; lo < r1; lo += C) {
     const uint32_t span = r1 - lo < C ? r1 - lo : C;
-    ++passes;
     const int4* const src = leaf ? a.out + S.pbase : v.stage_in;
     const uint32_t* const pidx = PICKLIKE ? a.out_idx + S.pbase : nullptr;
     PickArgs P;
@@ -1147,7 +1101,9 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       if (lay == kNarrow) acc_inner_sums<false>(src, v.stage_in_sum, total, lo, span);
       else acc_inner_sums<true>(src, v.stage_in_sum, total, lo, span);
     }
-    if (tid == 0) S.stage = stg;
+    if (!CLUSTER && tid == 0) S.stage = stg;
+    if (!waited) cluster_wait();
+    waited = true;
     __syncthreads();  // every update of the pass is done
     const unsigned long long at = S.stage + lo;
     if (PICKLIKE) {
@@ -1170,12 +1126,96 @@ __device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, 
       __syncthreads();
     }
   }
+  if (!waited) cluster_wait();
+}
+
+// Passes over the item's samples, the mark pass included (statistics).
+__device__ __forceinline__ uint32_t vox_passes(uint32_t C) {
+  const VoxShared& S = vox_shared();
+  return 1u + (S.r1 - S.r0 + C - 1u) / C;
+}
+
+}  // namespace
+
+// Voxelize one item (a child node c of an inner node p at level v.level):
+// all of its ranks, or, for a queued unit (r_unit, p_unit), the ranks
+// [D r / P, D (r + 1) / P) of its D occupied cells.  `first`: the item's
+// first attempt, which reserves the item's staging block (D records) and,
+// when its cells need several accumulate passes, may queue the ranges after
+// the first for the partition kernel.  The CTA that holds range 0 also
+// publishes what it reads (the leaf's points, the children's voxels).
+// `next_item` (first attempts): where thread 0 leaves the item the CTA
+// takes next, fetched while this one is marked.
+template <int MODE>
+__device__ __forceinline__ void vox_item(const BuildArgs& a, const VoxLevel& v, DevCounters* __restrict__ ctr, uint32_t it,
+                                         uint32_t r_unit, uint32_t p_unit, bool first, uint32_t* next_item) {
+  VoxShared& S = vox_shared();
+  uint4* const bits4 = reinterpret_cast<uint4*>(vox_smem);
+  const uint32_t tid = threadIdx.x;
+  vox_header(a, v, it);
+#pragma unroll
+  for (uint32_t i = 0; i < kWords / 4u / kVoxThreads; ++i) bits4[tid + i * kVoxThreads] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  constexpr bool WEIGHTED = MODE == LOD_WEIGHTED, PICKLIKE = MODE != LOD_FILTER && !WEIGHTED;  // one sample kept per cell
+  const bool leaf = S.I.leaf;
+  const bool lead = r_unit == 0;  // the one CTA of the item that publishes
+  const uint32_t total = leaf ? (uint32_t)S.I.n : S.cpre[S.nch];  // samples
+  // the next item's counter value; its latency hides behind the mark pass
+  uint32_t next_k = 0;
+  if (next_item && tid == 0) next_k = atomicAdd(&ctr->item_head, 1u);
+
+  if (WEIGHTED && tid < (uint32_t)__popc(S.pmask)) S.border[tid] = v.border[S.pfirst + tid];
+
+  // ---- pass 1: mark the occupied cells
+  if (!leaf) mark_inner<MODE == LOD_FILTER>(v.stage_in, 0u, total, lead ? v.dense : nullptr, v.dense_cap);
+  else if (a.wide) mark_wide(a.wide + 2 * S.pbase, total, lead ? a.out + S.pbase : nullptr, lead ? a.out_idx + S.pbase : nullptr);
+  else mark_leaf(a.out + S.pbase, total);
+  __syncthreads();
+
+  uint32_t next_it = next_k;
+  if (next_item && tid == 0 && v.order && next_k < v.n_items) next_it = v.order[next_k];
+  const uint32_t D = vox_rank_cells();
+  // the narrowest sums that provably cannot overflow for the points of this cube
+  const SumLayout lay = leaf && S.I.npts <= kLeafMaxSamples ? kLeaf16 : (S.I.npts <= kNarrowMaxSamples ? kNarrow : kWide);
+  const uint32_t cap = PICKLIKE ? kCapPick : WEIGHTED ? kCapWeighted : (lay == kLeaf16 ? kCapLeaf : (lay == kNarrow ? kCapNarrow : kCapWide));
+  const uint32_t C = (v.range_cells && v.range_cells < cap) ? v.range_cells : cap;  // ranks per pass
+  // thread 0: the item's first staging record.  The reservation (or, for
+  // a unit, the read of the first attempt's) is issued here and its value
+  // first used before the first extraction, so its latency overlaps the
+  // accumulate pass.
+  unsigned long long stg = 0;
+  if (tid == 0) {
+    S.D = D;
+    if (first) {
+      stg = atomicAdd(v.stage_used, (unsigned long long)D);
+      v.aux[S.I.g].occ = D;
+      S.r0 = 0;
+      S.r1 = D;
+      const uint32_t P = (D + C - 1) / C;
+      if (P > 1) atomicAdd(&ctr->vox_retries, 1ull);
+      uint32_t q0 = 0;
+      if (P > 1 && v.units && P >= v.queue_ranges && reserve_units(&ctr->units, v.unit_cap, P - 1, &q0)) {
+        for (uint32_t r = 1; r < P; ++r) v.units[q0 + r - 1] = make_uint4(it, r, P, 0u);
+        S.r1 = D / P;
+      }
+    } else {
+      stg = v.aux[S.I.g].stage;  // reserved by the first attempt
+      S.r0 = (uint32_t)((uint64_t)D * r_unit / p_unit);
+      S.r1 = (uint32_t)((uint64_t)D * (r_unit + 1) / p_unit);
+    }
+    S.n_wraps = 0;
+    S.settle = 0;
+  }
+  __syncthreads();
+
+  vox_ranges<MODE, false>(a, v, ctr, lay, C, stg);
   if (tid == 0) {
     if (first) {
       v.aux[S.I.g].stage = stg;
       if (stg + D > v.stage_cap) atomicOr(&ctr->error, kErrStageCap);
     }
     if (next_item) *next_item = next_it;  // read after this item's last barrier
+    const uint32_t passes = vox_passes(C);
     atomicAdd(&ctr->vox_passes, (unsigned long long)passes);
     atomicAdd(&ctr->vox_samples, (unsigned long long)passes * total);
     if (first) atomicMax(&ctr->vox_max_item, (unsigned long long)S.I.n);
@@ -1218,39 +1258,126 @@ __global__ void __launch_bounds__(kVoxThreads, kVoxCtasPerSm)
     __syncthreads();
     if (u >= n_units) break;
     const uint4 w = v.units[u];
-    vox_item<MODE>(a, v, ctr, w.x, w.y, w.z, false, nullptr, w.w != 0u);
+    vox_item<MODE>(a, v, ctr, w.x, w.y, w.z, false, nullptr);
   }
 }
 
-// Levels with few items (the top of the tree) would leave most SMs idle
-// with one CTA per item: every item is split up front into 2^m rank ranges
-// (its staging block reserved here, for as many cells as it can occupy)
-// and the partition kernel spreads them over the SMs.
-__global__ void k_vox_split(BuildArgs a, VoxLevel v, DevCounters* __restrict__ ctr, uint32_t m) {
-  const uint32_t it = blockIdx.x * blockDim.x + threadIdx.x;
-  if (it >= v.n_items) return;
-  const uint32_t t = find_tile(v.item_prefix, a.n_tiles, it);
-  const uint32_t* ls = v.lvl_start + (uint64_t)t * (kMaxLevels + 1);
-  const uint64_t g = a.tiles[t].node_base + ls[v.level + 1] + (it - v.item_prefix[t]);
-  const lod_node_t& c = v.nodes[g];
-  const uint64_t n = (c.flags & LOD_NODE_LEAF) ? c.point_count : c.voxel_count;
-  const uint64_t bound = umin64(n, kOctCells);
-  const unsigned long long base = atomicAdd(v.stage_used, (unsigned long long)bound);
-  if (base + bound > v.stage_cap) atomicOr(&ctr->error, kErrStageCap);
-  v.aux[g].stage = base;
-  v.aux[g].occ = 0u;
-  const uint32_t q = atomicAdd(&ctr->units, 1u << m);
-  if (q + (1u << m) > v.unit_cap) {
-    atomicOr(&ctr->error, kErrInternal);
-    return;
+namespace {
+
+// Shared-memory address of byte `off` of vox_smem in CTA `cta` of the cluster.
+__device__ __forceinline__ uint32_t far_addr(uint32_t off, uint32_t cta) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(vox_smem) + off), "r"(cta));
+  return a;
+}
+__device__ __forceinline__ uint4 far_ld4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+
+}  // namespace
+
+// Levels with few items (the top of the tree, the deepest levels): a cluster
+// of 2^lp CTAs takes an item.  Every CTA marks (and publishes) a share of the
+// samples in a bitmap of its own; each merges a slice of all the bitmaps and
+// collects the other slices, through distributed shared memory; then every
+// CTA ranks the merged bitmap and takes a part of the ranks, reading all of
+// the samples.
+//
+// Bound by the length of that chain for the largest item.  Measured against
+// units that each marked the whole item before they took a part of its ranks
+// (a launch to split the items and one for the units), and one CTA per item
+// above a quarter of the SMs: 1M points (56 and 8 items) 83 -> 57 us, 10M indoor
+// points first come (ten levels) 787 -> 602 us, 20M indoor points random (twelve)
+// 1160 -> 991 us, the root's 8 items of 500M points 172 -> 101 us.  (Adding each
+// CTA's share of the samples to the entries of the whole cluster by remote
+// atomics instead is slower for most levels, and atom.shared::cluster.min.u64
+// lost updates.)
+template <int MODE>
+__global__ void __launch_bounds__(kVoxThreads, 1)
+    k_vox_cluster(const __grid_constant__ BuildArgs a, const __grid_constant__ VoxLevel v, DevCounters* __restrict__ ctr, uint32_t lp) {
+  VoxShared& S = vox_shared();
+  constexpr bool WEIGHTED = MODE == LOD_WEIGHTED, PICKLIKE = MODE != LOD_FILTER && !WEIGHTED;
+  const uint32_t tid = threadIdx.x, parts = 1u << lp, part = blockIdx.x & (parts - 1u), k = blockIdx.x >> lp;
+  const uint32_t it = v.order ? v.order[k] : k;  // largest items first
+  uint4* const bits4 = reinterpret_cast<uint4*>(vox_smem);
+  vox_header(a, v, it);
+#pragma unroll
+  for (uint32_t i = 0; i < kWords / 4u / kVoxThreads; ++i) bits4[tid + i * kVoxThreads] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  const bool leaf = S.I.leaf;
+  const uint32_t total = leaf ? (uint32_t)S.I.n : S.cpre[S.nch];
+  const uint32_t first = (uint32_t)(((uint64_t)total * part) >> lp), end = (uint32_t)(((uint64_t)total * (part + 1u)) >> lp);
+  if (WEIGHTED && tid < (uint32_t)__popc(S.pmask)) S.border[tid] = v.border[S.pfirst + tid];
+
+  // ---- mark and publish the CTA's share
+  if (!leaf) mark_inner<MODE == LOD_FILTER>(v.stage_in, first, end, v.dense, v.dense_cap);
+  else if (a.wide) mark_wide(a.wide + 2 * (S.pbase + first), end - first, a.out + S.pbase + first, a.out_idx + S.pbase + first);
+  else mark_leaf(a.out + S.pbase + first, end - first);
+  cluster_arrive();
+  vox_clear_dense<MODE>();
+  cluster_wait();
+  // ---- merge: slice `part` of every CTA's bitmap into the own one ...
+  const uint32_t slice = (kWords / 4u) >> lp;  // in groups of four words
+  for (uint32_t i = tid; i < slice; i += kVoxThreads) {
+    const uint32_t at = part * slice + i;
+    uint4 w = bits4[at];
+    for (uint32_t q = 1; q < parts; ++q) {
+      const uint4 x = far_ld4(far_addr(16u * at, (part + q) & (parts - 1u)));
+      w.x |= x.x, w.y |= x.y, w.z |= x.z, w.w |= x.w;
+    }
+    bits4[at] = w;
   }
-  for (uint32_t j = 0; j < (1u << m); ++j) v.units[q + j] = make_uint4(it, j, 1u << m, 1u);
+  cluster_arrive();
+  cluster_wait();
+  // ---- ... then the other slices from the CTAs that merged them (which
+  // leave those alone from here on)
+  for (uint32_t i = tid; i < kWords / 4u; i += kVoxThreads) {
+    const uint32_t from = i / slice;
+    if (from != part) bits4[i] = far_ld4(far_addr(16u * i, from));
+  }
+  __syncthreads();
+  const uint32_t D = vox_rank_cells();
+  const SumLayout lay = leaf && S.I.npts <= kLeafMaxSamples ? kLeaf16 : (S.I.npts <= kNarrowMaxSamples ? kNarrow : kWide);
+  const uint32_t cap = PICKLIKE ? kCapPick : WEIGHTED ? kCapWeighted : (lay == kLeaf16 ? kCapLeaf : (lay == kNarrow ? kCapNarrow : kCapWide));
+  const uint32_t C = (v.range_cells && v.range_cells < cap) ? v.range_cells : cap;  // ranks per pass
+  if (tid == 0) {
+    S.D = D;
+    S.r0 = (uint32_t)(((uint64_t)D * part) >> lp);
+    S.r1 = (uint32_t)(((uint64_t)D * (part + 1u)) >> lp);
+    S.n_wraps = 0;
+    S.settle = 0;
+    if (part == 0) {
+      // the item's staging block, told to the other CTAs
+      const unsigned long long stg = atomicAdd(v.stage_used, (unsigned long long)D);
+      v.aux[S.I.g].occ = D;
+      v.aux[S.I.g].stage = stg;
+      if (stg + D > v.stage_cap) atomicOr(&ctr->error, kErrStageCap);
+      if (D > C << lp) atomicAdd(&ctr->vox_retries, 1ull);
+      for (uint32_t q = 0; q < parts; ++q)
+        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(far_addr(kSharedOff + (uint32_t)offsetof(VoxShared, stage), q)), "l"(stg)
+                     : "memory");
+    }
+  }
+  // waited for before the first extraction: by then every CTA has collected
+  // its slices (so any of them may leave) and knows the staging block
+  cluster_arrive();
+  __syncthreads();
+  vox_ranges<MODE, true>(a, v, ctr, lay, C, 0ull);
+  if (tid == 0) {
+    const uint32_t passes = vox_passes(C);
+    atomicAdd(&ctr->vox_passes, (unsigned long long)passes);
+    atomicAdd(&ctr->vox_samples, (unsigned long long)(passes - 1u) * total + (end - first));
+    if (part == 0) atomicMax(&ctr->vox_max_item, (unsigned long long)S.I.n);
+  }
 }
 
 template <int MODE>
 static void vox_attrs() {
   cudaFuncSetAttribute(k_vox<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   cudaFuncSetAttribute(k_vox_units<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  cudaFuncSetAttribute(k_vox_cluster<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
 }
 
 // One-time kernel attributes of the voxel pass (called before any launch,
@@ -1273,14 +1400,25 @@ int vox_init() {
 template <int MODE>
 static cudaError_t launch_vox_mode(const BuildArgs& a, const VoxLevel& v, DevCounters* ctr, cudaStream_t st) {
   const uint32_t ctas = (uint32_t)(vox_init() * kVoxCtasPerSm);
-  if (v.units && v.n_items * 4u <= ctas) {
-    uint32_t m = 0;
-    while (m < 3 && (v.n_items << (m + 1)) <= ctas) ++m;
-    k_vox_split<<<(v.n_items + 127) / 128, 128, 0, st>>>(a, v, ctr, m);
+  // few items: clusters of CTAs, as large as the SMs hold at once (another
+  // wave of clusters costs more than it shortens: 56 items in clusters of 8
+  // took 3 times as long as one CTA each)
+  const uint32_t lp = v.n_items * 8u <= ctas ? 3u : v.n_items * 4u <= ctas ? 2u : v.n_items * 2u <= ctas ? 1u : 0u;
+  if (lp) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1u << lp;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(v.n_items << lp);
+    cfg.blockDim = dim3(kVoxThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_vox_cluster<MODE>, a, v, ctr, lp);
     note_launch();
-    k_vox_units<MODE><<<ctas, kVoxThreads, kSmemBytes, st>>>(a, v, ctr);
-    note_launch();
-    return cudaGetLastError();
+    return e;
   }
   k_vox<MODE><<<v.n_items < ctas ? v.n_items : ctas, kVoxThreads, kSmemBytes, st>>>(a, v, ctr);
   note_launch();

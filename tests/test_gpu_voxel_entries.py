@@ -119,3 +119,25 @@ def test_weighted_samples_across_octants(lod, L, depth):
     pts[:, :3] = p
     pts[:, 3] = rng.integers(-(2**31), 2**31, n)
     check(lod, pts, 20, 2, max_depth=depth)
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5, 9, 10])
+def test_levels_of_few_items(lod, mode, tiles):
+    # 8 to 80 items at the top level: clusters of 8, 4 and 2 CTAs, and none;
+    # leaves (with kept indices) and inner children beside each other
+    import torch
+    rng = np.random.default_rng(17 * tiles + mode)
+    clouds = []
+    for t in range(tiles):
+        n = 9001 + 700 * t
+        pts = np.empty((n, 4), np.int32)
+        pts[:, :3] = rng.integers(0, 1 << 12, (n, 3))
+        pts[: n // 3, :3] >>= 2
+        pts[:2, :3] = [[0, 0, 0], [(1 << 12) - 1] * 3]
+        pts[:, 3] = rng.integers(-(2**31), 2**31, n)
+        clouds.append(pts)
+    rs = lod.build_batched([torch.from_numpy(c).cuda() for c in clouds], 1500, mode, keep_index=True)
+    for c, r in zip(clouds, rs):
+        compare(r.to_host(), oracle.build(c, 1500, mode, 21), inp=c)
+        r.free()
