@@ -1036,7 +1036,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     LOD_CK(d_aux.alloc(total_cap * sizeof(NodeAux)));
     LOD_LAUNCH("nodes", 0,
                launch_nodes(A, d_nodes.as<lod_node_t>(), d_aux.as<NodeAux>(), g_lvl, g_nn, g_rb->leaf_cap, &g_rb->nctr,
-                            refined, st));
+                            refined, total_cap, st));
     return LOD_OK;
   };
   bool nodes_enqueued = false;

@@ -884,7 +884,8 @@ cudaError_t launch_scatter(const BuildArgs& a, const uint32_t* chunk_src, const 
 
 // ---------------------------------------------------------------- node table
 // Breadth-first node list (Section 4.1.3 creates the node list from the
-// count pyramid): one CTA per tile walks the levels; a node is split iff it
+// count pyramid): `parts` CTAs per tile (one, or a cluster of kNodeParts)
+// walk the levels, a CTA's worth of nodes per CTA and step; a node is split iff it
 // holds more than T points, is above max_depth and larger than a unit cube.
 // Children are the non-empty octants in octant order, their counts read
 // from the pyramid of the grid that covers them (switching to the
@@ -893,27 +894,43 @@ cudaError_t launch_scatter(const BuildArgs& a, const uint32_t* chunk_src, const 
 // right after the first round and that round created refinement grids, the
 // table would have to follow later rounds anyway, so the pass stands down
 // at once (the host builds the table after the last round).
+//
+// Bound by a step's chain of dependent reads and by the record stores of the
+// SMs that take part.  Measured, one CTA against a cluster of eight: 500M indoor
+// points 507 -> 192 us, 200M 243 -> 151 us, 12M aerial points (T 3000) 131 -> 97 us.
+
+constexpr uint32_t kNodeParts = 8;
+
+// A cluster-wide barrier; what the CTAs wrote before it, in global memory and
+// in each other's shared memory, is visible after it.
+__device__ __forceinline__ void node_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __restrict__ nodes,
                                                   NodeAux* __restrict__ aux, uint32_t* __restrict__ lvl_start,
                                                   uint32_t* __restrict__ n_nodes,
                                                   unsigned long long* __restrict__ leaf_cap,
                                                   DevCounters* __restrict__ ctr,
-                                                  const unsigned long long* __restrict__ refined) {
+                                                  const unsigned long long* __restrict__ refined, uint32_t parts) {
+  const uint32_t t = blockIdx.x / parts, part = blockIdx.x - t * parts;
   if (a.abort && *a.abort) return;
   if (refined && *refined) {
-    if (threadIdx.x == 0) n_nodes[blockIdx.x] = kNone;
+    if (threadIdx.x == 0 && part == 0) n_nodes[t] = kNone;
     return;
   }
   __shared__ uint32_t warp_sum[32];
   __shared__ uint32_t s_total;
-  __shared__ int s_fail;
-  const uint32_t t = blockIdx.x;
+  __shared__ uint32_t s_fail;
+  // children (and, above, the failure code) of every CTA's nodes of a step; two
+  // steps' worth, since a CTA may still read a step's when another writes the next's
+  __shared__ uint32_t s_part[2][kNodeParts];
   const TileDesc td = a.tiles[t];
   lod_node_t* nd = nodes + td.node_base;
   NodeAux* ax = aux + td.node_base;
   uint32_t* ls = lvl_start + (uint64_t)t * (kMaxLevels + 1);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0) s_fail = 0;
+  if (threadIdx.x == 0 && part == 0) {
     lod_node_t r;
     const SrcDesc& rs = a.srcs[t];  // the tile's first counting grid covers the root cube
     r.min[0] = rs.min[0];
@@ -934,16 +951,16 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
     ax[0].src = t;
     ax[0].j = 0;
     ax[0].c = 0;
-    s_fail = 0;
   }
-  __syncthreads();
-  uint32_t begin = 0, end = 1, level = 0;
+  if (parts > 1) node_cluster_sync();  // every CTA has started; the root is in place
+  else __syncthreads();
+  uint32_t begin = 0, end = 1, level = 0, step = 0, fail = 0;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   while (begin < end) {
-    if (threadIdx.x == 0) ls[level] = begin;
+    if (threadIdx.x == 0 && part == 0) ls[level] = begin;
     uint32_t next = end;
-    for (uint32_t chunk = begin; chunk < end; chunk += blockDim.x) {
-      const uint32_t i = chunk + threadIdx.x;
+    for (uint32_t chunk = begin; chunk < end; chunk += parts * blockDim.x, ++step) {
+      const uint32_t i = chunk + part * blockDim.x + threadIdx.x;
       const bool valid = i < end;
       uint32_t mask = 0, cc[8];
       uint32_t sid = 0, j = 0, c = 0;
@@ -965,7 +982,7 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
           const uint32_t child = a.srcs[sid].map[c];
           if (a.srcs[child].cnt == nullptr) {
             split = false;
-            s_fail = 2;
+            s_fail = 2u;
           } else {
             sid = child;
             j = 0;
@@ -1007,9 +1024,48 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
         if (lane == nw - 1) s_total = wi;
       }
       __syncthreads();
-      const uint32_t pos = warp_sum[warp] + incl - nch;
-      const uint32_t total = s_total;
+      uint32_t pos = warp_sum[warp] + incl - nch;
+      uint32_t total = s_total, before = 0;  // children of the step's nodes, of the CTAs before this one
+      fail = s_fail;
+      if (parts > 1) {
+        if (threadIdx.x < parts) {
+          uint32_t at;
+          asm("mapa.shared::cluster.u32 %0, %1, %2;"
+              : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_part[step & 1u][part])), "r"(threadIdx.x));
+          asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(total | (fail << 16)) : "memory");
+        }
+        node_cluster_sync();
+        total = 0;
+        for (uint32_t q = 0; q < parts; ++q) {
+          const uint32_t v = s_part[step & 1u][q];
+          if (q == part) before = total;
+          total += v & 0xFFFFu;
+          fail |= v >> 16;
+        }
+      }
       const bool fits = (uint64_t)next + total <= td.node_cap;
+      pos += before;
+      // per level: bound on the voxel records the nodes' octants can contribute
+      // to their parents (all nodes), and the exact leaf points.  In a large
+      // tree one atomic a warp; in a small one the reductions would lengthen
+      // every level by more than the atomics, which nothing waits for
+      if (fits && parts == 1 && valid) {
+        atomicAdd(&leaf_cap[level], (unsigned long long)umin64(cnt, kOctCells));
+        if (!split) atomicAdd(&leaf_cap[kMaxLevels + 1 + level], (unsigned long long)cnt);
+        else atomicAdd(&leaf_cap[2 * (kMaxLevels + 1)], (unsigned long long)umin64(cnt, kVoxelGuess));
+      }
+      if (fits && parts > 1) {
+        const uint32_t occ = __reduce_add_sync(0xFFFFFFFFu, valid ? (uint32_t)umin64(cnt, kOctCells) : 0u);
+        const uint32_t guess = __reduce_add_sync(0xFFFFFFFFu, split ? (uint32_t)umin64(cnt, kVoxelGuess) : 0u);
+        uint64_t pts = valid && !split ? cnt : 0;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) pts += __shfl_xor_sync(0xFFFFFFFFu, pts, o);
+        if (lane == 0) {
+          if (occ) atomicAdd(&leaf_cap[level], (unsigned long long)occ);
+          if (pts) atomicAdd(&leaf_cap[kMaxLevels + 1 + level], (unsigned long long)pts);
+          if (guess) atomicAdd(&leaf_cap[2 * (kMaxLevels + 1)], (unsigned long long)guess);
+        }
+      }
       if (valid && fits) {
         const SrcDesc& sd = a.srcs[sid];
         const uint32_t st = sd.start[pyr_off(j) + c];
@@ -1018,11 +1074,6 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
         nd[i].child_mask = (uint8_t)mask;
         nd[i].flags = split ? 0 : (LOD_NODE_LEAF | (cnt > a.T ? LOD_NODE_OVERFULL : 0));
         nd[i].first_child = split ? next + pos : kNone;
-        // per level: bound on the voxel records the node's octant can
-        // contribute to its parent (all nodes), and the exact leaf points
-        atomicAdd(&leaf_cap[lvl], (unsigned long long)umin64(cnt, kOctCells));
-        if (!split) atomicAdd(&leaf_cap[kMaxLevels + 1 + lvl], (unsigned long long)cnt);
-        else atomicAdd(&leaf_cap[2 * (kMaxLevels + 1)], (unsigned long long)umin64(cnt, kVoxelGuess));
         if (split) {
           const uint32_t half = lg - 1;
           uint32_t r = 0;
@@ -1053,30 +1104,49 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
           }
         }
       }
-      if (!fits && threadIdx.x == 0) s_fail = 1;
+      if (!fits) fail |= 1u;
       next += total;
       __syncthreads();
-      if (s_fail) break;
+      if (fail) break;
     }
-    if (s_fail) break;
+    if (fail) break;
+    if (parts > 1) node_cluster_sync();  // the next level's records are in place
     begin = end;
     end = next;
     ++level;
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && part == 0) {
     ls[level] = begin;
     for (uint32_t l = level + 1; l <= kMaxLevels; ++l) ls[l] = begin;
-    n_nodes[t] = s_fail ? kNone : end;
-    if (s_fail == 1) atomicOr(&ctr->error, kErrNodeCap);
+    n_nodes[t] = fail ? kNone : end;
+    if (fail & 1u) atomicOr(&ctr->error, kErrNodeCap);
   }
 }
 
 cudaError_t launch_nodes(const BuildArgs& a, lod_node_t* nodes, NodeAux* aux, uint32_t* lvl_start,
                          uint32_t* n_nodes, unsigned long long* leaf_cap, DevCounters* ctr,
-                         const unsigned long long* refined, cudaStream_t st) {
-  k_nodes<<<a.n_tiles, kBlock, 0, st>>>(a, nodes, aux, lvl_start, n_nodes, leaf_cap, ctr, refined);
+                         const unsigned long long* refined, uint64_t node_cap, cudaStream_t st) {
+  // A cluster per tile while all of them run at once (16 clusters of 8) and the
+  // tables have room for 32768 nodes a tile on average (16 per leaf_threshold
+  // points, so 2044 times that many points).  Below, most levels fit one CTA
+  // and a cluster's barriers cost more than its stores save: one tile's table,
+  // one CTA against a cluster, at 400 times leaf_threshold points 62 and 89
+  // us, at 1000 times 43 and 55 us, at 4000 times 131 and 97 us (aerial) or
+  // 243 and 151 us (indoor), at 10,000 times 507 and 192 us.
+  const uint32_t parts = a.n_tiles <= 16u && node_cap >= 32768ull * a.n_tiles ? kNodeParts : 1u;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = parts;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.n_tiles * parts);
+  cfg.blockDim = dim3(kBlock);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = parts > 1 ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_nodes, a, nodes, aux, lvl_start, n_nodes, leaf_cap, ctr, refined, parts);
   note_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace lodk

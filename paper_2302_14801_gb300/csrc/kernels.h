@@ -29,7 +29,7 @@ cudaError_t launch_scatter(const BuildArgs& a, const uint32_t* chunk_src, const 
                            uint32_t round, int grid, cudaStream_t st);
 cudaError_t launch_nodes(const BuildArgs& a, lod_node_t* nodes, NodeAux* aux, uint32_t* lvl_start,
                          uint32_t* n_nodes, unsigned long long* leaf_cap, DevCounters* ctr,
-                         const unsigned long long* refined, cudaStream_t st);
+                         const unsigned long long* refined, uint64_t node_cap, cudaStream_t st);
 
 // ----- voxel sampling (Section 4.2) -----
 struct VoxLevel {
@@ -60,7 +60,7 @@ struct VoxLevel {
   uint64_t border_cap;
   ulonglong2* root_sums;  // filtered: exact sums of the top level's voxels, parallel to dense (or null)
   // rank ranges: an item whose occupied cells need P >= queue_ranges
-  // accumulate passes hands ranges 1..P-1 to the partition kernel (0xFFFFFFFF:
+  // accumulate passes hands ranges 1..P-1 to the units launch (0xFFFFFFFF:
   // never); range_cells (nonzero) caps the cells of one pass below what the
   // shared memory holds
   uint32_t queue_ranges;
