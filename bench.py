@@ -214,10 +214,10 @@ def cpu_oracle_sample(cloud, T: int, budget_s: float = 12.0) -> dict:
 # the dominant one (the roofline below stays HBM: the path has no dense
 # contraction and no other measured peak applies).
 LIMITERS = {
-    "voxelize": "shared-memory pipe, over half of it atomics (ncu: short-scoreboard stalls, 0.6-0.7 shared "
-                "wavefronts per active SM cycle, DRAM 3-6 % on the 20M cut)",
-    "scatter": "scattered stores and load latency (ncu: long-scoreboard stalls, DRAM 45 %, 36 % L2 write hits)",
-    "count": "instruction issue (ncu: 68 % issue active, DRAM 41 %)",
+    "voxelize": "shared-memory pipe, issue and barriers (ncu: short-scoreboard and barrier stalls, 40 % issue "
+                "active, DRAM 4-21 % on the 20M cut)",
+    "scatter": "scattered stores and load latency (ncu: long-scoreboard stalls, DRAM 45 %, 21 % L2 write hits)",
+    "count": "load latency and instruction issue (ncu: 59 % issue active, DRAM 41 %)",
     "bbox": "HBM bandwidth",
 }
 

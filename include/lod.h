@@ -336,10 +336,11 @@ int lod_root_cubes_noalloc(const lod_point_t* const* d_tiles, const uint64_t* n,
  *                   8; default 4096).
  *   vox_queue_ranges  the voxel pass numbers an item's occupied cells in
  *                   cell order and accumulates them in ranges of what one
- *                   CTA's shared memory holds (5120 to 10240 cells); an
+ *                   CTA's shared memory holds (4688 to 17817 cells); an
  *                   item needing P >= vox_queue_ranges ranges hands ranges
  *                   2..P to other SMs (default 4; 1: every range stays with
- *                   the item's CTA; at most 4096).
+ *                   the item's CTA; at most 4096).  Levels of so few items
+ *                   that SMs would idle share every item between SMs anyway.
  *   graph_voxel_levels  1: every build captures the launches of all its
  *                   voxel levels (which need no host round trip between
  *                   them) into one CUDA graph and launches that (0: plain

@@ -126,8 +126,8 @@ struct DevCounters {
   unsigned long long vox_max_item;    // samples of the level's largest item (statistics)
   unsigned long long border_used;     // weighted mode: entries of the level's border lists
   unsigned int error;                 // nonzero: a kernel detected a problem
-  unsigned int units;                 // voxel partition units queued this level
-  unsigned int unit_head;             // units taken by the partition kernel
+  unsigned int units;                 // rank ranges of voxel items queued this level
+  unsigned int unit_head;             // of them, taken by the units launch
   unsigned int item_head;             // items taken by the first-attempt kernel
 };
 

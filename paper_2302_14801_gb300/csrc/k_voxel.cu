@@ -33,8 +33,8 @@
 // data pipe (43 %, half of it the atomics' bank and address conflicts) and
 // the barriers between an item's phases.  Measured against 64-bit atomic
 // sums merged over equal lanes and 128-bit compare-and-swap picks (all levels
-// of one build, GB300): 500M indoor points filtered 11.5 -> 8.4 ms, 50M
-// aerial filtered 1.14 -> 0.74 ms, 200M indoor points picked 5.9 -> 5.5 ms.
+// of one build, GB300): 500M indoor points filtered 11.5 -> 8.2 ms, 50M
+// aerial filtered 1.14 -> 0.72 ms, 200M indoor points picked 5.9 -> 5.4 ms.
 //
 // Every octant's voxels go to a staging area; a level scan then assigns
 // each parent one contiguous voxel range (children are consecutive in node
@@ -254,8 +254,7 @@ __device__ __forceinline__ bool reserve_units(unsigned int* count, uint32_t cap,
 }
 
 // Everything a voxel CTA keeps in shared memory is one dynamic array, so that
-// the phases below (separate functions: each gets the registers for itself)
-// address it as shared memory.
+// the phases below address it as shared memory.
 extern __shared__ __align__(16) unsigned char vox_smem[];
 
 namespace {
@@ -1142,7 +1141,7 @@ __device__ __forceinline__ uint32_t vox_passes(uint32_t C) {
 // [D r / P, D (r + 1) / P) of its D occupied cells.  `first`: the item's
 // first attempt, which reserves the item's staging block (D records) and,
 // when its cells need several accumulate passes, may queue the ranges after
-// the first for the partition kernel.  The CTA that holds range 0 also
+// the first for k_vox_units.  The CTA that holds range 0 also
 // publishes what it reads (the leaf's points, the children's voxels).
 // `next_item` (first attempts): where thread 0 leaves the item the CTA
 // takes next, fetched while this one is marked.
