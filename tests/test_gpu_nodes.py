@@ -39,3 +39,12 @@ def test_capacity_overflow(lod):  # noqa: F811
     pts[:, :3] = xyz
     pts[:, 3] = np.arange(len(xyz))
     compare(gpu_build(lod, pts, T, 0), oracle.build(pts, T, 0), inp=pts)
+
+
+def test_uneven_tiles(lod):  # noqa: F811
+    import torch
+    tiles = [_cube(n, 17, n) for n in (150_000, 1, 90_000)]  # a cluster each, the one-point tile's too
+    rs = lod.build_batched([torch.from_numpy(t).cuda() for t in tiles], 2, 0)
+    for t, r in zip(tiles, rs):
+        compare(r.to_host(), oracle.build(t, 2, 0, 21), inp=t)
+        r.free()
