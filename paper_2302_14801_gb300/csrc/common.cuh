@@ -18,9 +18,9 @@ constexpr uint32_t kRootMaxD = 8;      // depth of the largest first counting gr
 constexpr uint32_t kSmemBins = 4096;   // grids up to 8^4 bins are counted in shared memory
 constexpr uint32_t kOctCells = 1u << 18;  // 64^3 cells of one child octant (Section 4.2)
 constexpr uint32_t kBlock = 1024;
-// Voxels of an inner node, for the first size of the voxel array: as many as
-// its points, or what a surface crossing a 128^3 grid occupies (16,000 to
-// 20,000 cells measured on the aerial cloud).
+// Voxels of an inner node of two children or more, for the first size of the
+// voxel array: as many as its points, or what a surface crossing a 128^3 grid
+// occupies (16,000 to 20,000 cells measured on the aerial cloud).
 constexpr uint64_t kVoxelGuess = 20480;
 
 // Offset of level j inside a count/start pyramid stored level by level

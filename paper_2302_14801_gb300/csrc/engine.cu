@@ -629,6 +629,15 @@ bool keeps_index(const lod_params_t& p) {
   return p.mode == LOD_PICK || p.mode == LOD_FIRST || p.mode == LOD_RANDOM || (p.flags & LOD_FLAG_LEAF_INDEX);
 }
 
+// Most records that the voxel array of a build of n points starts with: half
+// the points, or 20480 voxels (about a surface through a node's grid) per
+// leaf_threshold points, since clouds have 0.35 to 1.06 inner nodes per
+// leaf_threshold points, but no more than four a point (leaves of 200 to 3000
+// points give 0.9 to 3.7 voxels a point).
+static uint64_t first_voxels(uint64_t n, uint64_t T) {
+  return std::max<uint64_t>({n / 2, 4096, (uint64_t)((double)n * std::min(4.0, (double)kVoxelGuess / (double)T))});
+}
+
 uint64_t estimate_result_bytes(uint64_t n, const lod_params_t& p) {
   const bool idx = keeps_index(p);
   const uint64_t T = std::max<uint32_t>(p.leaf_threshold, 1);
@@ -917,7 +926,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   struct NodeRead {
     DevCounters ctr, nctr;
     // [0, L): per level sum over all nodes of min(points, 64^3); [L, 2L): exact
-    // leaf points; [2L]: about how many voxels the inner nodes have
+    // leaf points; [2L]: about how many voxels the inner nodes have (those of two children or more)
     unsigned long long leaf_cap[2 * (kMaxLevels + 1) + 1];
     unsigned int abort, pad;
   };
@@ -1274,10 +1283,13 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   DevCounters* const g_lctr = reinterpret_cast<DevCounters*>(d_vread.as<char>() + vr_ctr);
   unsigned long long* const g_tvox = reinterpret_cast<unsigned long long*>(d_vread.as<char>() + vr_tvox);
   // the voxel array's first size: half the points is ample for leaves of
-  // tens of thousands of points, but small leaves give up to 2.5 voxels a
+  // tens of thousands of points, but small leaves give up to 3.7 voxels a
   // point, and an array found too small costs a second run of the levels
-  // (12M aerial points, leaves of 3000: 3.2 -> 2.2 ms a build)
-  uint64_t dense_cap = std::max<uint64_t>({M / 2, 4096, leaf_cap[2 * (kMaxLevels + 1)]});
+  // (12M aerial points, leaves of 3000: 3.2 -> 2.2 ms a build).  The sum over
+  // the nodes is not bounded by the cloud (nodes above one another count the
+  // same points), so it is held to what clouds need at most
+  uint64_t dense_cap =
+      std::max<uint64_t>({M / 2, 4096, std::min<uint64_t>(leaf_cap[2 * (kMaxLevels + 1)], first_voxels(M, T))});
   std::vector<DevCounters> lctr(std::max(n_vlev, 1));
   unsigned long long vstate[2] = {0, 0};
   std::vector<unsigned long long> tvox(nt);

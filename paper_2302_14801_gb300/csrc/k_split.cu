@@ -1046,17 +1046,21 @@ __global__ void __launch_bounds__(kBlock) k_nodes(BuildArgs a, lod_node_t* __res
       const bool fits = (uint64_t)next + total <= td.node_cap;
       pos += before;
       // per level: bound on the voxel records the nodes' octants can contribute
-      // to their parents (all nodes), and the exact leaf points.  In a large
-      // tree one atomic a warp; in a small one the reductions would lengthen
-      // every level by more than the atomics, which nothing waits for
+      // to their parents (all nodes), and the exact leaf points; over all levels,
+      // about how many voxels the inner nodes have (without those of a single
+      // child, which has their voxels too: a chain would count the same points at
+      // every level).  In a large tree one atomic a warp; in a small one the
+      // reductions would lengthen every level by more than the atomics, which
+      // nothing waits for
+      const bool fork = split && nch > 1;
       if (fits && parts == 1 && valid) {
         atomicAdd(&leaf_cap[level], (unsigned long long)umin64(cnt, kOctCells));
         if (!split) atomicAdd(&leaf_cap[kMaxLevels + 1 + level], (unsigned long long)cnt);
-        else atomicAdd(&leaf_cap[2 * (kMaxLevels + 1)], (unsigned long long)umin64(cnt, kVoxelGuess));
+        else if (fork) atomicAdd(&leaf_cap[2 * (kMaxLevels + 1)], (unsigned long long)umin64(cnt, kVoxelGuess));
       }
       if (fits && parts > 1) {
         const uint32_t occ = __reduce_add_sync(0xFFFFFFFFu, valid ? (uint32_t)umin64(cnt, kOctCells) : 0u);
-        const uint32_t guess = __reduce_add_sync(0xFFFFFFFFu, split ? (uint32_t)umin64(cnt, kVoxelGuess) : 0u);
+        const uint32_t guess = __reduce_add_sync(0xFFFFFFFFu, fork ? (uint32_t)umin64(cnt, kVoxelGuess) : 0u);
         uint64_t pts = valid && !split ? cnt : 0;
 #pragma unroll
         for (int o = 16; o; o >>= 1) pts += __shfl_xor_sync(0xFFFFFFFFu, pts, o);

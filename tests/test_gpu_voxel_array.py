@@ -1,0 +1,93 @@
+"""Size of the voxel array: its first size is held to a few records a point on
+clouds whose nodes stand above one another, where the number of voxels cannot
+be told from the node counts."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import oracle
+from compare import compare
+
+pytestmark = pytest.mark.gpu
+
+NODE, POINT, VOXEL = 56, 16, 16
+
+
+@pytest.fixture(scope="module")
+def lod():
+    import torch
+    from paper_2302_14801_gb300 import _build_ext
+    _build_ext.build()
+    from paper_2302_14801_gb300 import lod as m
+    torch.cuda.set_device(0)
+    return m
+
+
+class Pool:
+    """The device's default stream-ordered pool, which holds the results."""
+    USED, USED_HIGH = 7, 8  # cudaMemPoolAttrUsedMemCurrent, cudaMemPoolAttrUsedMemHigh
+
+    def __init__(self):
+        import torch
+        try:
+            self.rt = ctypes.CDLL("libcudart.so.13")
+        except OSError:
+            pytest.skip("CUDA runtime library not found by name")
+        self.pool = ctypes.c_void_p()
+        assert self.rt.cudaDeviceGetDefaultMemPool(ctypes.byref(self.pool), torch.cuda.current_device()) == 0
+
+    def read(self, attr):
+        val = ctypes.c_uint64()
+        assert self.rt.cudaMemPoolGetAttribute(self.pool, attr, ctypes.byref(val)) == 0
+        return val.value
+
+    def peak_of(self, call):
+        """What call() returns, and the most bytes in use meanwhile beyond those before."""
+        import torch
+        torch.cuda.synchronize()
+        zero = ctypes.c_uint64(0)
+        assert self.rt.cudaMemPoolSetAttribute(self.pool, self.USED_HIGH, ctypes.byref(zero)) == 0
+        base = self.read(self.USED)
+        out = call()
+        torch.cuda.synchronize()
+        return out, self.read(self.USED_HIGH) - base
+
+
+def clusters(n, each, chain):
+    """Clusters of `each` points, identical ones, or (chain) identical but for a
+    point at 1, 2, 4 ... from them, so that every node above has two children."""
+    rng = np.random.default_rng(n + each)
+    k = n // each
+    at = rng.choice(1 << 18, k, replace=False)
+    base = np.stack([at & 63, (at >> 6) & 63, at >> 12], 1) << 16
+    xyz = np.repeat(base[:, None], each, axis=1)
+    if chain:
+        xyz[:, :16, 0] += 1 << np.arange(16)
+    pts = np.empty((n, 4), np.int32)
+    pts[:, :3] = xyz.reshape(-1, 3)
+    pts[:, 3] = rng.integers(-(2**31), 2**31, n)
+    return pts
+
+
+def first_voxels(n, T):
+    return max(n // 2, 4096, int(n * min(4.0, 20480 / T)))
+
+
+@pytest.mark.parametrize("chain", [False, True])
+@pytest.mark.parametrize("T,each", [(1000, 5000), (20_000, 50_000)])
+def test_first_size_is_a_few_records_a_point(lod, T, each, chain):
+    import torch
+    n = 1_000_000
+    pts = clusters(n, each, chain)
+    d = torch.from_numpy(pts).cuda()
+    want = oracle.build(pts, T, 0)
+    r, peak = Pool().peak_of(lambda: lod.build(d, T, 0))
+    got = r.to_host()
+    r.free()
+    compare(got, want, inp=pts)
+    nodes = 64 + 16 * -(-n // T)
+    while nodes < len(want["level"]):
+        nodes *= 4
+    # the result at the array's first size, its trimmed copy, and 1 MB for rounding
+    assert peak <= n * POINT + nodes * NODE + (first_voxels(n, T) + len(want["voxels"])) * VOXEL + (1 << 20)
