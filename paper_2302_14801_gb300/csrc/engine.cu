@@ -1288,8 +1288,9 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   // (12M aerial points, leaves of 3000: 3.2 -> 2.2 ms a build).  The sum over
   // the nodes is not bounded by the cloud (nodes above one another count the
   // same points), so it is held to what clouds need at most
+  const uint64_t dense_least = std::max<uint64_t>(M / 2, 4096);
   uint64_t dense_cap =
-      std::max<uint64_t>({M / 2, 4096, std::min<uint64_t>(leaf_cap[2 * (kMaxLevels + 1)], first_voxels(M, T))});
+      std::max<uint64_t>(dense_least, std::min<uint64_t>(leaf_cap[2 * (kMaxLevels + 1)], first_voxels(M, T)));
   std::vector<DevCounters> lctr(std::max(n_vlev, 1));
   unsigned long long vstate[2] = {0, 0};
   std::vector<unsigned long long> tvox(nt);
@@ -1303,8 +1304,20 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       "voxelize_L30", "voxelize_L31", "voxelize_L32", "voxelize_L33"};
   DevBuf d_rsums(st);  // result (out-of-core merges): exact sums of the roots' voxels
   for (int attempt = 0;; ++attempt) {
-    LOD_CK(d_dense.alloc(dense_cap * 16));
-    if (opt.keep_root_sums && filt) LOD_CK(d_rsums.alloc(dense_cap * 16));
+    // no memory for the generous first size: half the points, and a second
+    // run if that is too small
+    auto alloc_dense = [&]() -> cudaError_t {
+      const cudaError_t e = d_dense.alloc(dense_cap * 16);
+      return e == cudaSuccess && opt.keep_root_sums && filt ? d_rsums.alloc(dense_cap * 16) : e;
+    };
+    cudaError_t de = alloc_dense();
+    if (de == cudaErrorMemoryAllocation && attempt == 0 && dense_cap > dense_least) {
+      (void)cudaGetLastError();
+      d_dense.release();
+      dense_cap = dense_least;
+      de = alloc_dense();
+    }
+    LOD_CK(de);
     LOD_CK(cudaMemsetAsync(d_vread.p, 0, vr_bytes, st));
     // optionally, every level's launches go into one CUDA graph (the
     // levels need no host round trip, so they can be captured as a unit)

@@ -1,6 +1,7 @@
 """Size of the voxel array: its first size is held to a few records a point on
 clouds whose nodes stand above one another, where the number of voxels cannot
-be told from the node counts."""
+be told from the node counts; a build that has no memory for it makes do with
+less."""
 import ctypes
 
 import numpy as np
@@ -8,6 +9,7 @@ import pytest
 
 import oracle
 from compare import compare
+from paper_2302_14801_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -91,3 +93,42 @@ def test_first_size_is_a_few_records_a_point(lod, T, each, chain):
         nodes *= 4
     # the result at the array's first size, its trimmed copy, and 1 MB for rounding
     assert peak <= n * POINT + nodes * NODE + (first_voxels(n, T) + len(want["voxels"])) * VOXEL + (1 << 20)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_no_memory_for_the_first_size(lod, mode, monkeypatch):
+    # the k-th device allocation of the build fails (on the host, never asked of
+    # CUDA).  The voxel array's first one, here more than half a record a point,
+    # is asked for again with less; the ones before it are not, nor are the picked
+    # points after it
+    import torch
+    pts = synth.indoor(400_000, seed=41, n_prims=64)
+    want = oracle.build(pts, 3000, mode, 21)
+    assert len(want["voxels"]) > len(pts) // 2  # the levels run twice with less
+    d = torch.from_numpy(pts).cuda()
+    pool, built = Pool(), []
+    lod.build(d, 3000, mode).free()
+    torch.cuda.synchronize()
+    base = pool.read(Pool.USED)
+    for k in range(1, 64):
+        monkeypatch.setenv("LOD_INJECT_OOM_AT", str(k))
+        try:
+            r = lod.build(d, 3000, mode, full_precision=mode == 1)
+        except lod.LodError as e:
+            assert e.status == lod.LOD_ERR_OOM
+            torch.cuda.synchronize()
+            assert pool.read(Pool.USED) == base
+            continue
+        monkeypatch.delenv("LOD_INJECT_OOM_AT")
+        built.append(k)
+        compare(r.to_host(), want, inp=pts)
+        r.free()
+    first = built[0]
+    if mode == 1:
+        assert built[1] > first + 1  # a later failure is a failure
+    monkeypatch.setenv("LOD_INJECT_OOM_AT", str(first))
+    r = lod.build(d, 3000, mode)
+    monkeypatch.delenv("LOD_INJECT_OOM_AT")
+    nodes = r.device_bytes() - len(pts) * (POINT + 4 * mode) - len(want["voxels"]) * VOXEL
+    r.free()
+    assert nodes in [(64 + 16 * 134) * NODE * 4**j for j in range(3)]  # the second run left the exact size
