@@ -1398,6 +1398,27 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       continue;
     }
     if (vstate[1]) return LOD_ERR_INTERNAL;
+    // Trim an array found too large (a copy of the voxels): half a record a
+    // point is kept up to three times its need, since its slack costs little;
+    // a first size above that, whose slack would be several records a point,
+    // up to one and a half times.
+    const uint64_t V = vstate[0];
+    if (dense_cap > (dense_cap > dense_least ? V + V / 2 : 3 * V) + 65536 && !d_rsums.p) {
+      DevBuf exact(st);
+      const cudaError_t e = exact.alloc(std::max<uint64_t>(V, 1) * 16);
+      if (e == cudaErrorMemoryAllocation && attempt == 0 && dense_cap > dense_least) {
+        // no room for both: the levels once more, into an array of the exact size
+        (void)cudaGetLastError();
+        dense_cap = std::max<uint64_t>(V, 1);
+        prof.resolve();
+        continue;
+      }
+      LOD_CK(e);
+      if (V) LOD_CK(cudaMemcpyAsync(exact.p, d_dense.p, V * 16, cudaMemcpyDeviceToDevice, st));
+      std::swap(exact.p, d_dense.p);
+      std::swap(exact.bytes, d_dense.bytes);
+      dense_cap = std::max<uint64_t>(V, 1);
+    }
     break;
   }
   const uint64_t V = vstate[0];
@@ -1438,22 +1459,12 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
                  launch_unwide(A, d_units.as<uint32_t>(), (uint32_t)leaf_roots.size(), max_n, st));
     }
   }
-  // trim the voxel array when the estimate was more than three times too
-  // generous (a copy of the voxels; smaller slack is cheaper to keep)
-  if (dense_cap > 3 * V + 65536 && !d_rsums.p) {
-    DevBuf exact(st);
-    LOD_CK(exact.alloc(std::max<uint64_t>(V, 1) * 16));
-    if (V) LOD_CK(cudaMemcpyAsync(exact.p, d_dense.p, V * 16, cudaMemcpyDeviceToDevice, st));
-    std::swap(exact.p, d_dense.p);
-    std::swap(exact.bytes, d_dense.bytes);
-    dense_cap = std::max<uint64_t>(V, 1);
-  }
   // full-precision variant: the picked input points, parallel to the voxels
   DevBuf d_vpts(st);  // result
   if ((prm.flags & LOD_FLAG_FULL_PRECISION) && V) {
     uint32_t max_nodes = 0;
     for (uint32_t t = 0; t < nt; ++t) max_nodes = std::max(max_nodes, n_nodes[t]);
-    LOD_CK(d_vpts.alloc(dense_cap * 16));
+    LOD_CK(d_vpts.alloc(V * 16));
     LOD_LAUNCH("voxel_points", 32.0 * V,
                launch_voxel_points(g_tiles, nt, d_nodes.as<lod_node_t>(), g_nn, max_nodes, V,
                                    d_dense.as<int4>(), d_vpts.as<int4>(), st));
@@ -1473,7 +1484,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     r.n_voxels = tvox[t];
   }
   sh->bytes = M * 16 + (want_idx ? M * 4 : 0) + total_cap * sizeof(lod_node_t) + dense_cap * 16 +
-              (d_vpts.p ? dense_cap * 16 : 0);
+              (d_vpts.p ? V * 16 : 0);
   sh->voxel_points = d_vpts.take();
   if (d_rsums.p) sh->bytes += dense_cap * 16;
   sh->root_sums = d_rsums.take();

@@ -99,8 +99,8 @@ def test_first_size_is_a_few_records_a_point(lod, T, each, chain):
 def test_no_memory_for_the_first_size(lod, mode, monkeypatch):
     # the k-th device allocation of the build fails (on the host, never asked of
     # CUDA).  The voxel array's first one, here more than half a record a point,
-    # is asked for again with less; the ones before it are not, nor are the picked
-    # points after it
+    # is asked for again with less, and its trimmed copy done without; the ones
+    # before them are not, nor are the picked points after them
     import torch
     pts = synth.indoor(400_000, seed=41, n_prims=64)
     want = oracle.build(pts, 3000, mode, 21)
@@ -125,10 +125,27 @@ def test_no_memory_for_the_first_size(lod, mode, monkeypatch):
         r.free()
     first = built[0]
     if mode == 1:
-        assert built[1] > first + 1  # a later failure is a failure
+        assert built != list(range(first, 64))  # a later failure is a failure
     monkeypatch.setenv("LOD_INJECT_OOM_AT", str(first))
     r = lod.build(d, 3000, mode)
     monkeypatch.delenv("LOD_INJECT_OOM_AT")
     nodes = r.device_bytes() - len(pts) * (POINT + 4 * mode) - len(want["voxels"]) * VOXEL
     r.free()
     assert nodes in [(64 + 16 * 134) * NODE * 4**j for j in range(3)]  # the second run left the exact size
+
+
+@pytest.mark.parametrize("cloud,T", [("indoor", 3000), ("indoor", 1000), ("aerial", 3000), ("sphere", 1000)])
+@pytest.mark.parametrize("full", [False, True])
+def test_results_keep_little_slack(lod, cloud, T, full):
+    # a result holds at most half a record a point, or half as many more records
+    # than voxels (and 65536, below which nothing is copied); its picked points
+    # at full precision are as many as its voxels
+    import torch
+    n = 3_000_000
+    pts = getattr(synth, cloud)(n, seed=1)
+    r = lod.build(torch.from_numpy(pts).cuda(), T, 1 if full else 0, full_precision=full)
+    v = r.view().n_voxels
+    extra = r.device_bytes() - n * (POINT + 4 * full) - v * VOXEL * full
+    r.free()
+    nodes = 64 + 16 * -(-n // T)
+    assert extra <= nodes * NODE + max(n // 2, v + v // 2 + 65536) * VOXEL
