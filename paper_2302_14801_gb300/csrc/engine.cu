@@ -1302,20 +1302,16 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       "voxelize_L18", "voxelize_L19", "voxelize_L20", "voxelize_L21", "voxelize_L22", "voxelize_L23",
       "voxelize_L24", "voxelize_L25", "voxelize_L26", "voxelize_L27", "voxelize_L28", "voxelize_L29",
       "voxelize_L30", "voxelize_L31", "voxelize_L32", "voxelize_L33"};
-  DevBuf d_rsums(st);  // result (out-of-core merges): exact sums of the roots' voxels
+  VoxLevel vl;
+  std::memset(&vl, 0, sizeof(vl));
   for (int attempt = 0;; ++attempt) {
     // no memory for the generous first size: half the points, and a second
     // run if that is too small
-    auto alloc_dense = [&]() -> cudaError_t {
-      const cudaError_t e = d_dense.alloc(dense_cap * 16);
-      return e == cudaSuccess && opt.keep_root_sums && filt ? d_rsums.alloc(dense_cap * 16) : e;
-    };
-    cudaError_t de = alloc_dense();
+    cudaError_t de = d_dense.alloc(dense_cap * 16);
     if (de == cudaErrorMemoryAllocation && attempt == 0 && dense_cap > dense_least) {
       (void)cudaGetLastError();
-      d_dense.release();
       dense_cap = dense_least;
-      de = alloc_dense();
+      de = d_dense.alloc(dense_cap * 16);
     }
     LOD_CK(de);
     LOD_CK(cudaMemsetAsync(d_vread.p, 0, vr_bytes, st));
@@ -1328,8 +1324,6 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       LOD_CK(cap.begin());
     }
     const cudaStream_t vst = use_graph ? cap.cap : st;  // where the levels are enqueued
-    VoxLevel vl;
-    std::memset(&vl, 0, sizeof(vl));
     for (int l = n_vlev - 1; l >= 0; --l) {
       const uint32_t* ip = &pref[(size_t)l * pstride];
       const uint32_t n_items = ip[nt], n_par = ip[nt + 1 + nt];
@@ -1376,9 +1370,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     if (n_vlev > 0) {
       // the roots' voxels: the items of the top level have no parent pass
       // that would copy their staged records
-      vl.root_sums = d_rsums.as<ulonglong2>();
       LOD_LAUNCH("publish_top", 0, launch_copy_items(A, vl, vst));
-      vl.root_sums = nullptr;
     }
     if (use_graph) LOD_CK(cap.launch());
     char* const hv = static_cast<char*>(tl_stage.get(vr_bytes));
@@ -1403,7 +1395,7 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     // a first size above that, whose slack would be several records a point,
     // up to one and a half times.
     const uint64_t V = vstate[0];
-    if (dense_cap > (dense_cap > dense_least ? V + V / 2 : 3 * V) + 65536 && !d_rsums.p) {
+    if (dense_cap > (dense_cap > dense_least ? V + V / 2 : 3 * V) + 65536) {
       DevBuf exact(st);
       const cudaError_t e = exact.alloc(std::max<uint64_t>(V, 1) * 16);
       if (e == cudaErrorMemoryAllocation && attempt == 0 && dense_cap > dense_least) {
@@ -1440,6 +1432,16 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       V_child = lv;
     }
     if (prof.on && n_vlev > 0 && !prof.recs.empty()) prof.recs.back().bytes = 32.0 * (double)V_child;
+  }
+  // the exact sums of the roots' voxels (the last of the array), for
+  // out-of-core merges, while the top level's staging still holds them
+  DevBuf d_rsums(st);  // result
+  const uint64_t top_voxels = n_vlev > 0 ? lctr[0].level_voxels : 0;
+  if (opt.keep_root_sums && filt && n_vlev > 0) {
+    LOD_CK(d_rsums.alloc(std::max<uint64_t>(top_voxels, 1) * 16));
+    vl.root_sums = d_rsums.as<ulonglong2>();
+    vl.root_base = V - top_voxels;
+    LOD_LAUNCH("root_sums", 0, launch_root_sums(A, vl, st));
   }
   if (A.wide) {
     // a root that is a leaf is no voxel item: publish its points here
@@ -1486,8 +1488,9 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   sh->bytes = M * 16 + (want_idx ? M * 4 : 0) + total_cap * sizeof(lod_node_t) + dense_cap * 16 +
               (d_vpts.p ? V * 16 : 0);
   sh->voxel_points = d_vpts.take();
-  if (d_rsums.p) sh->bytes += dense_cap * 16;
+  if (d_rsums.p) sh->bytes += top_voxels * 16;
   sh->root_sums = d_rsums.take();
+  sh->root_base = V - top_voxels;
   sh->points = d_points.take();
   sh->index = want_idx ? d_index.take() : nullptr;
   sh->nodes = d_nodes.take();

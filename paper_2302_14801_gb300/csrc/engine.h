@@ -19,7 +19,9 @@ struct SharedBuffers {
   void* nodes = nullptr;    // node tables of all tiles
   void* voxels = nullptr;   // voxels of all tiles
   void* voxel_points = nullptr;  // full-precision picked points, parallel to voxels (or null)
-  void* root_sums = nullptr;     // BuildOptions::keep_root_sums: packed exact sums parallel to voxels
+  void* root_sums = nullptr;     // BuildOptions::keep_root_sums: packed exact sums of the roots' voxels,
+                                 // which start at record root_base of voxels
+  uint64_t root_base = 0;
   void* input = nullptr;    // owned copy of host input (lod_build_from_host), or null
   uint64_t bytes = 0;
   ~SharedBuffers();

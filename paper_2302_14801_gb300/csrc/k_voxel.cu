@@ -1558,11 +1558,9 @@ __global__ void __launch_bounds__(256) k_copy_items(BuildArgs a, VoxLevel v) {
                      (it - v.item_prefix[t]);
   const NodeAux ca = v.aux[g];
   if (ca.dense + ca.occ > v.dense_cap) return;  // the build is redone with a larger array
-  const bool filt = a.mode == LOD_FILTER;  // records may carry their sums packed
+  const bool filt = a.mode == LOD_FILTER;  // records may carry their sums packed, which are not published
   for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < ca.occ; i += gridDim.y * blockDim.x) {
     int4 rec = v.stage_out[ca.stage + i];
-    const bool packed = filt && (uint32_t)rec.w != kNone;
-    if (v.root_sums) v.root_sums[ca.dense + i] = packed ? unpack_sums(rec) : v.stage_out_sum[ca.stage + i];
     if (filt) rec.w = (int)kNone;
     v.dense[ca.dense + i] = rec;
   }
@@ -1571,6 +1569,27 @@ __global__ void __launch_bounds__(256) k_copy_items(BuildArgs a, VoxLevel v) {
 cudaError_t launch_copy_items(const BuildArgs& a, const VoxLevel& v, cudaStream_t st) {
   if (!v.n_items) return cudaSuccess;
   k_copy_items<<<dim3(v.n_items, v.n_items <= 64 ? 32u : 4u), 256, 0, st>>>(a, v);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// The exact sums of those voxels, of which the staged records or the sums array
+// behind them hold one each (out-of-core batches only, after the levels).
+__global__ void __launch_bounds__(256) k_root_sums(BuildArgs a, VoxLevel v) {
+  const uint32_t it = blockIdx.x;
+  const uint32_t t = find_tile(v.item_prefix, a.n_tiles, it);
+  const NodeAux ca = v.aux[a.tiles[t].node_base + v.lvl_start[(uint64_t)t * (kMaxLevels + 1) + v.level + 1] +
+                           (it - v.item_prefix[t])];
+  for (uint32_t i = threadIdx.x; i < ca.occ; i += blockDim.x) {
+    const int4 rec = v.stage_out[ca.stage + i];
+    v.root_sums[ca.dense - v.root_base + i] =
+        (uint32_t)rec.w != kNone ? unpack_sums(rec) : v.stage_out_sum[ca.stage + i];
+  }
+}
+
+cudaError_t launch_root_sums(const BuildArgs& a, const VoxLevel& v, cudaStream_t st) {
+  if (!v.n_items) return cudaSuccess;
+  k_root_sums<<<v.n_items, 256, 0, st>>>(a, v);
   note_launch();
   return cudaGetLastError();
 }

@@ -58,7 +58,8 @@ struct VoxLevel {
   uint4* border;
   int4* border_list;
   uint64_t border_cap;
-  ulonglong2* root_sums;  // filtered: exact sums of the top level's voxels, parallel to dense (or null)
+  ulonglong2* root_sums;  // launch_root_sums: where the exact sums of the top level's voxels go
+  uint64_t root_base;     // ... the first of which is record root_base of dense
   // rank ranges: an item whose occupied cells need P >= queue_ranges
   // accumulate passes hands ranges 1..P-1 to the units launch (0xFFFFFFFF:
   // never); range_cells (nonzero) caps the cells of one pass below what the
@@ -75,6 +76,8 @@ cudaError_t launch_level_scan(const BuildArgs& a, const VoxLevel& v, const uint3
                               uint32_t n_parents, unsigned long long* tile_voxels, DevCounters* ctr,
                               cudaStream_t st);
 cudaError_t launch_copy_items(const BuildArgs& a, const VoxLevel& v, cudaStream_t st);
+// Filtered mode, top level: its voxels' exact sums, from the staged records.
+cudaError_t launch_root_sums(const BuildArgs& a, const VoxLevel& v, cudaStream_t st);
 cudaError_t launch_unwide(const BuildArgs& a, const uint32_t* tiles, uint32_t n_tiles, uint32_t max_points,
                           cudaStream_t st);
 cudaError_t launch_voxel_points(const TileDesc* tiles, uint32_t n_tiles, const lod_node_t* nodes,

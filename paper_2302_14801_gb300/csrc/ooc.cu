@@ -440,7 +440,7 @@ int build_out_of_core(const lod_point_t* h, uint64_t n, const lod_params_t& prm,
               S.kind = 0;
             } else {
               S.recs = static_cast<const int4*>(b.voxels) + root.voxel_offset;
-              S.sums = b.root_sums ? static_cast<const ulonglong2*>(b.root_sums) + root.voxel_offset : nullptr;
+              S.sums = b.root_sums ? static_cast<const ulonglong2*>(b.root_sums) + (root.voxel_offset - b.root_base) : nullptr;
               S.n = root.voxel_count;
               S.kind = 1;
             }

@@ -149,3 +149,22 @@ def test_results_keep_little_slack(lod, cloud, T, full):
     r.free()
     nodes = 64 + 16 * -(-n // T)
     assert extra <= nodes * NODE + max(n // 2, v + v // 2 + 65536) * VOXEL
+
+
+def test_out_of_core_batches_keep_little(lod):
+    # eight chunks in several batches, whose arrays all stay until the merge of
+    # the root: a first size of four records a point must not stay with them,
+    # nor sums beside it
+    n, T, batch = 1_000_000, 1000, 250_000
+    pts = clusters(n, 5000, True)
+    want = oracle.build(pts, T, 0)
+    r, peak = Pool().peak_of(lambda: lod.build_out_of_core(pts, T, 0, 21, chunk_points=n // 2, stream_points=batch, batch_points=batch))
+    compare(r.to_host(), want, inp=pts)
+    r.free()
+    nodes = 8 * 64 + 16 * (n // T + 8)
+    # every chunk's points, nodes and voxels with their sums, one batch's input
+    # (points and indices) and first size, the counts of the top grid's 256^3
+    # cells, the merge's grid (40 bytes for each of 128^3 cells), the assembled result
+    most = (2 * (n * POINT + nodes * NODE + len(want["voxels"]) * 2 * VOXEL)
+            + batch * (POINT + 4) + first_voxels(batch, T) * VOXEL + 4 * 256**3 + 40 * 128**3)
+    assert peak <= most + (4 << 20)
