@@ -1260,14 +1260,18 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       LOD_CK(d_sum1.alloc(stage_cap * 16));
     }
   }
-  // weighted mode: the border lists of one level (no more entries than the
-  // level's items have samples)
+  // weighted mode: the border lists of one level.  An entry is a sample of one
+  // of its items, a point or a voxel that stands for one of the item's points
+  // or more: no more than the level's leaf points and min(points, 64^3) of its
+  // inner nodes (one layer of voxels along each middle plane, 3 * 128^2, is
+  // below 64^3), and no more than the cloud's points
   const bool weighted = prm.mode == LOD_WEIGHTED;
   DevBuf d_border(st, ws), d_blist(st, ws);
   uint64_t border_cap = 0;
   if (weighted && n_vlev > 0) {
     for (int l = 0; l < n_vlev; ++l)
       border_cap = std::max<uint64_t>(border_cap, leaf_cap[kMaxLevels + 1 + l + 1] + leaf_cap[l + 1]);
+    border_cap = std::min<uint64_t>(border_cap, M);
     LOD_CK(d_border.alloc(total_cap * sizeof(uint4)));
     LOD_CK(d_blist.alloc(border_cap * sizeof(int4)));
   }
