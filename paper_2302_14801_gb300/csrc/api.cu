@@ -385,7 +385,8 @@ struct Request {
   const lod_point_t* d_points = nullptr;
   uint64_t n = 0;
   lod_params_t params;
-  uint64_t est = 0;
+  uint64_t est = 0;    // the build's footprint
+  uint64_t extra = 0;  // and what it takes more if its voxel array may start generous
   bool done = false;
   int status = LOD_NOT_READY;
   lod_result_t* result = nullptr;
@@ -417,8 +418,12 @@ struct lod_server {
     for (;;) {
       std::shared_ptr<Request> rq;
       bool trim = false;
+      lodk::BuildOptions opt;
+      opt.exact_voxel_array = true;
       {
-        // admission: FIFO head, once it fits into what the budget has left
+        // admission: FIFO head, once it fits into what the budget has left;
+        // its voxel array starts generous (so that its levels run once) if
+        // that fits as well
         std::unique_lock<std::mutex> lk(budget->mu);
         for (;;) {
           {
@@ -429,6 +434,8 @@ struct lod_server {
               if (budget->in_use + need <= budget->limit) {
                 rq = h;
                 queue.pop_front();
+                opt.small_voxel_array = budget->in_use + need + rq->extra > budget->limit;
+                if (!opt.small_voxel_array) need += rq->extra;
                 budget->in_use += need;
                 blocked = 0;
               } else if (ws_acc && ++blocked >= 2) {
@@ -463,7 +470,7 @@ struct lod_server {
       lodk::TileInput ti{rq->d_points, rq->n};
       std::shared_ptr<lodk::SharedBuffers> sh;
       std::vector<lodk::TileResult> tr;
-      int rc = lodk::run_build(&ti, 1, rq->params, st, &sh, &tr, nullptr);
+      int rc = lodk::run_build(&ti, 1, rq->params, st, &sh, &tr, nullptr, true, opt);
       lod_result_t* res = nullptr;
       if (rc == LOD_OK) {
         res = make_result(sh, tr[0], rq->params.mode, sh->bytes);
@@ -531,6 +538,7 @@ int lod_submit(lod_server_t* s, const lod_point_t* d_points, uint64_t n, const l
   rq->params = params ? *params : defaults();
   if (!lodk::valid_params(rq->params)) return LOD_ERR_INVALID_ARG;
   rq->est = lodk::estimate_build_bytes(n, rq->params);
+  rq->extra = lodk::estimate_voxel_array_bytes(n, rq->params);
   if (rq->est > s->budget->limit) return LOD_ERR_BUDGET;
   {
     std::lock_guard<std::mutex> lk(s->mu);

@@ -652,13 +652,22 @@ uint64_t estimate_build_bytes(uint64_t n, const lod_params_t& p) {
   const uint64_t nodes = 64 + 16 * ((n + T - 1) / T);
   // result + one refinement buffer + two staging levels of one record per
   // point (plus exact sums when filtering, plus the border lists when
-  // weighting) + the voxel array's first
-  // estimate + node aux + pool, plus the 32-byte leaf staging of modes that
-  // keep input indices
+  // weighting) + as much again as the result's half a voxel record per point
+  // (an array of that size and its trimmed copy, or the picked points) + node
+  // aux + pool, plus the 32-byte leaf staging of modes that keep input indices
   const bool keep_idx = keeps_index(p);
   const uint64_t staging = n * (p.mode == LOD_FILTER ? 64 : (p.mode == LOD_WEIGHTED ? 48 : 32));
   return estimate_result_bytes(n, p) + n * 20 + staging + n * 8 + (keep_idx ? n * 32 : 0) +
          nodes * sizeof(NodeAux) + pool + (16u << 20);
+}
+
+uint64_t estimate_voxel_array_bytes(uint64_t n, const lod_params_t& p) {
+  // the first size beside its trimmed copy, which is made of less than two
+  // thirds of it, or (full precision) beside the picked points; one record a
+  // point is charged by estimate_build_bytes
+  const uint64_t first = first_voxels(n, std::max<uint32_t>(p.leaf_threshold, 1));
+  const uint64_t most = (p.flags & LOD_FLAG_FULL_PRECISION) ? 2 * first : first + 2 * (first / 3);
+  return first > std::max<uint64_t>(n / 2, 4096) && most > n ? (most - n) * 16 : 0;
 }
 
 // Keep freed blocks of the device's stream-ordered pool instead of returning
@@ -1293,8 +1302,9 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
   // the nodes is not bounded by the cloud (nodes above one another count the
   // same points), so it is held to what clouds need at most
   const uint64_t dense_least = std::max<uint64_t>(M / 2, 4096);
-  uint64_t dense_cap =
-      std::max<uint64_t>(dense_least, std::min<uint64_t>(leaf_cap[2 * (kMaxLevels + 1)], first_voxels(M, T)));
+  uint64_t dense_cap = dense_least;
+  if (!opt.small_voxel_array)
+    dense_cap = std::max<uint64_t>(dense_cap, std::min<uint64_t>(leaf_cap[2 * (kMaxLevels + 1)], first_voxels(M, T)));
   std::vector<DevCounters> lctr(std::max(n_vlev, 1));
   unsigned long long vstate[2] = {0, 0};
   std::vector<unsigned long long> tvox(nt);
@@ -1397,9 +1407,10 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
     // Trim an array found too large (a copy of the voxels): half a record a
     // point is kept up to three times its need, since its slack costs little;
     // a first size above that, whose slack would be several records a point,
-    // up to one and a half times.
+    // up to one and a half times (not at all where results are counted).
     const uint64_t V = vstate[0];
-    if (dense_cap > (dense_cap > dense_least ? V + V / 2 : 3 * V) + 65536) {
+    const uint64_t kept = dense_cap <= dense_least ? 3 * V + 65536 : opt.exact_voxel_array ? V : V + V / 2 + 65536;
+    if (dense_cap > kept) {
       DevBuf exact(st);
       const cudaError_t e = exact.alloc(std::max<uint64_t>(V, 1) * 16);
       if (e == cudaErrorMemoryAllocation && attempt == 0 && dense_cap > dense_least) {

@@ -55,6 +55,10 @@ struct TileInput {
 
 struct BuildOptions {
   bool keep_root_sums = false;  // filtered mode: keep the exact sums of every root's voxels
+  // builds whose memory is counted (the server's): the voxel array starts at
+  // half a record a point; the result keeps no slack in one that is larger
+  bool small_voxel_array = false;
+  bool exact_voxel_array = false;
 };
 
 // Runs the complete build of n_tiles independent tiles on stream st.
@@ -77,8 +81,10 @@ void release_thread_arena();
 bool valid_params(const lod_params_t& p);
 bool keeps_index(const lod_params_t& p);
 
-// Rough device footprint (bytes) of building n points (result + temporaries).
+// Rough device footprint (bytes) of building n points (result + temporaries)
+// with BuildOptions::small_voxel_array, and what a build without it takes more.
 uint64_t estimate_build_bytes(uint64_t n, const lod_params_t& params);
+uint64_t estimate_voxel_array_bytes(uint64_t n, const lod_params_t& params);
 // Rough device footprint of a finished result of n points.
 uint64_t estimate_result_bytes(uint64_t n, const lod_params_t& params);
 

@@ -168,3 +168,61 @@ def test_out_of_core_batches_keep_little(lod):
     most = (2 * (n * POINT + nodes * NODE + len(want["voxels"]) * 2 * VOXEL)
             + batch * (POINT + 4) + first_voxels(batch, T) * VOXEL + 4 * 256**3 + 40 * 128**3)
     assert peak <= most + (4 << 20)
+
+
+def test_server_keeps_to_its_budget(lod):
+    # the smallest budget that takes the request leaves half a record a point for
+    # the voxel array; a large one lets it start at four, and the result keeps
+    # no slack either way
+    import torch
+    n, T = 1_000_000, 1000
+    pts = clusters(n, 5000, True)
+    d = torch.from_numpy(pts).cuda()
+    want = oracle.build(pts, T, 0)
+    nodes = 64 + 16 * (n // T)
+
+    def serve(budget):
+        srv = lod.Server(hbm_budget_bytes=budget, max_inflight=1)
+        try:
+            try:
+                ticket = srv.submit(d, T, 0)
+            except lod.LodError as e:
+                assert e.status == lod.LOD_ERR_BUDGET
+                return None
+            return srv.wait(ticket)
+        finally:
+            srv.close()
+
+    refused, taken = 1 << 20, 1 << 30
+    assert serve(refused) is None
+    while taken - refused > 1:
+        mid = (refused + taken) // 2
+        r = serve(mid)
+        if r is None:
+            refused = mid
+        else:
+            taken = mid
+            r.free()
+    for budget, records in ((taken, n // 2), (8 << 30, first_voxels(n, T))):
+        r, peak = Pool().peak_of(lambda: serve(budget))
+        compare(r.to_host(), want, inp=pts)
+        size = r.device_bytes()
+        r.free()
+        assert size == n * POINT + nodes * NODE + len(want["voxels"]) * VOXEL
+        assert peak <= n * POINT + nodes * NODE + (records + len(want["voxels"])) * VOXEL + (1 << 20)
+
+
+@pytest.mark.parametrize("cloud", ["indoor", "sphere"])
+def test_server_results_keep_no_slack(lod, cloud):
+    import torch
+    n, T = 1_000_000, 1000
+    d = torch.from_numpy(getattr(synth, cloud)(n, seed=1)).cuda()
+    srv = lod.Server(hbm_budget_bytes=8 << 30, max_inflight=1)
+    try:
+        r = srv.wait(srv.submit(d, T, 0))
+        v = r.view().n_voxels
+        assert v > n // 2
+        assert r.device_bytes() == n * POINT + (64 + 16 * (n // T)) * NODE + v * VOXEL
+        r.free()
+    finally:
+        srv.close()
