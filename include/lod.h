@@ -254,8 +254,8 @@ const char* lod_error_string(int status);
  * has no counterpart (its buffers are allocated once, Section 4.1.6).
  * lod_scratch_bytes: device bytes the workspace of `stream` holds now.
  * lod_trim: waits for `stream` to finish its work, frees its workspace and the
- *   calling thread's page-locked upload memory (at most 8 MB per thread), and
- *   returns the pool's unused memory to the device.  Results stay valid;
+ *   calling thread's page-locked upload and read-back memory (at most 8 MB each
+ *   per thread), and returns the pool's unused memory to the device.  Results stay valid;
  *   the next build on the stream allocates its scratch again.  A workspace
  *   that a build on another thread is using at that moment is left alone.
  *   Returns LOD_ERR_CUDA if the synchronisation reports an error. */

@@ -195,21 +195,23 @@ struct DevBuf {
   }
 };
 
-// Pinned host staging for read-backs, one per host thread.
+// Pinned host staging for read-backs, one per host thread, kept and given
+// back like the upload arena below (a batch's tile tables take 144 bytes a tile).
 struct HostStage {
   void* p = nullptr;
   size_t bytes = 0;
-  ~HostStage() {
+  ~HostStage() { release(); }
+  void release() {
     if (p) cudaFreeHost(p);
+    p = nullptr;
+    bytes = 0;
   }
   void* get(size_t b) {
     if (b > bytes) {
-      if (p) cudaFreeHost(p);
-      bytes = std::max<size_t>(b, 1 << 16);
-      if (cudaMallocHost(&p, bytes) != cudaSuccess) {
-        p = nullptr;
-        bytes = 0;
-      }
+      release();
+      const size_t cap = std::max<size_t>(b, 1 << 16);
+      if (cudaMallocHost(&p, cap) == cudaSuccess) bytes = cap;
+      else p = nullptr;
     }
     return p;
   }
@@ -249,6 +251,7 @@ struct Uploader {
     cudaStreamSynchronize(st);
     for (char* r : retired) cudaFreeHost(r);
     if (ar.cap > kArenaKeep) ar.release();
+    if (tl_stage.bytes > kArenaKeep) tl_stage.release();
   }
   cudaError_t put(void* dst, const void* src, size_t bytes) {
     if (!bytes) return cudaSuccess;
@@ -521,7 +524,11 @@ void release_workspace(cudaStream_t st) {
 }
 
 
-void release_thread_arena() { tl_arena.release(); }
+void release_thread_arena() {
+  tl_arena.release();
+  tl_stage.release();
+  if (debug_stats()) std::fprintf(stderr, "[lod] trim: page-locked bytes %zu\n", tl_arena.cap + tl_stage.bytes);
+}
 
 uint32_t default_root_depth(uint64_t n, uint32_t T, uint32_t max_depth) {
   if (n <= T || max_depth == 0 || T == 0) return 0;
@@ -703,8 +710,8 @@ struct PhaseClock {
   }
   ~PhaseClock() {
     if (on)
-      std::fprintf(stderr, "[lod] host ms:%s | total %.3f\n", line.c_str(),
-                   std::chrono::duration<double, std::milli>(last - t0).count());
+      std::fprintf(stderr, "[lod] host ms:%s | total %.3f | page-locked bytes %zu\n", line.c_str(),
+                   std::chrono::duration<double, std::milli>(last - t0).count(), tl_arena.cap + tl_stage.bytes);
   }
 };
 

@@ -73,7 +73,7 @@ int run_build(const TileInput* tiles, uint32_t n_tiles, const lod_params_t& para
 // (the stream must be idle).
 uint64_t workspace_bytes(cudaStream_t st);
 void release_workspace(cudaStream_t st);
-// Give back the calling thread's page-locked upload memory.
+// Give back the calling thread's page-locked upload and read-back memory.
 void release_thread_arena();
 
 // Parameter checks shared by every entry point, and whether a build keeps
