@@ -1396,13 +1396,22 @@ int vox_init() {
   return sms;
 }
 
+// A level's items are shared by clusters of 2^share_log2 CTAs: levels of few
+// items, by as many CTAs as the SMs hold at once (another wave of clusters
+// costs more than it shortens: 56 items in clusters of 8 took 3 times as long as
+// one CTA each).
+static constexpr uint32_t share_log2(uint32_t n_items, uint32_t ctas) {
+  return n_items <= ctas / 8u ? 3u : n_items <= ctas / 4u ? 2u : n_items <= ctas / 2u ? 1u : 0u;
+}
+static_assert(share_log2(19, 152) == 3 && share_log2(20, 152) == 2 && share_log2(38, 152) == 2 &&
+              share_log2(39, 152) == 1 && share_log2(76, 152) == 1 && share_log2(77, 152) == 0, "one wave of clusters");
+static_assert(share_log2(1u << 29, 152) == 0 && share_log2(1u << 30, 152) == 0 && share_log2(1u << 31, 152) == 0,
+              "no wrap at levels of 2^29 items and more");
+
 template <int MODE>
 static cudaError_t launch_vox_mode(const BuildArgs& a, const VoxLevel& v, DevCounters* ctr, cudaStream_t st) {
   const uint32_t ctas = (uint32_t)(vox_init() * kVoxCtasPerSm);
-  // few items: clusters of CTAs, as large as the SMs hold at once (another
-  // wave of clusters costs more than it shortens: 56 items in clusters of 8
-  // took 3 times as long as one CTA each)
-  const uint32_t lp = v.n_items * 8u <= ctas ? 3u : v.n_items * 4u <= ctas ? 2u : v.n_items * 2u <= ctas ? 1u : 0u;
+  const uint32_t lp = share_log2(v.n_items, ctas);
   if (lp) {
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
