@@ -159,21 +159,6 @@ struct DevBuf {
     bytes = b;
     return cudaMallocAsync(&p, b, st);
   }
-  // grow keeping the first `keep` bytes
-  cudaError_t grow(size_t b, size_t keep) {
-    if (b <= bytes) return cudaSuccess;
-    DevBuf q(st, ws);
-    cudaError_t e = q.alloc(b);
-    if (e != cudaSuccess) return e;
-    if (p && keep) {
-      e = cudaMemcpyAsync(q.p, p, std::min(keep, bytes), cudaMemcpyDeviceToDevice, st);
-      if (e != cudaSuccess) return e;
-    }
-    std::swap(p, q.p);
-    std::swap(bytes, q.bytes);
-    std::swap(blk, q.blk);
-    return cudaSuccess;
-  }
   void release() {
     if (p) {
       if (blk >= 0) ws->blocks[blk].used = false;
@@ -1411,10 +1396,13 @@ static int run_build_impl(const TileInput* tin, uint32_t nt, const lod_params_t&
       continue;
     }
     if (vstate[1]) return LOD_ERR_INTERNAL;
-    // Trim an array found too large (a copy of the voxels): half a record a
-    // point is kept up to three times its need, since its slack costs little;
-    // a first size above that, whose slack would be several records a point,
-    // up to one and a half times (not at all where results are counted).
+    // Trim an array found too large: half a record a point is kept up to three
+    // times its need; a first size above that, whose slack would be records
+    // for every point, up to one and a half times (not at all where results
+    // are counted).  The copy costs what it moves, two records a voxel: 23M
+    // indoor points, leaves of 2826, array 2.3 times the voxels: 4.21 -> 4.43
+    // ms; clouds whose array is less than 1.5 times the voxels (aerial, sphere
+    // with small leaves) pay nothing.
     const uint64_t V = vstate[0];
     const uint64_t kept = dense_cap <= dense_least ? 3 * V + 65536 : opt.exact_voxel_array ? V : V + V / 2 + 65536;
     if (dense_cap > kept) {

@@ -19,7 +19,7 @@
 // No hashing and no probing: every lookup costs the same, D is exact before
 // anything is accumulated (so the item's staging block is reserved to the
 // record), and the voxels come out sorted by cell.  The dense entries of
-// one pass hold 5939 to 17817 cells, depending on the layout; an item with
+// one pass hold 4688 to 17817 cells, depending on the layout; an item with
 // more occupied cells takes its ranks in consecutive ranges, one accumulate
 // pass each, and may hand ranges to other SMs.  Colour sums are exact
 // integers in 32-bit words (16-bit fields whose wraps are listed, 32-bit
@@ -29,12 +29,13 @@
 // Listing 1) keep, per cell, the smallest key by a 64-bit atomicMin, which is
 // native, and the colour of the sample that holds it.
 //
-// What bounds it: instruction issue (45 % of the slots), the shared-memory
-// data pipe (43 %, half of it the atomics' bank and address conflicts) and
-// the barriers between an item's phases.  Measured against 64-bit atomic
-// sums merged over equal lanes and 128-bit compare-and-swap picks (all levels
-// of one build, GB300): 500M indoor points filtered 11.5 -> 8.2 ms, 50M
-// aerial filtered 1.14 -> 0.72 ms, 200M indoor points picked 5.9 -> 5.4 ms.
+// What bounds it: the shared-memory data pipe (0.43 wavefronts per active SM
+// cycle in the largest level of 20M indoor points, 43 % of them the atomics'),
+// instruction issue (40 % of the slots) and the barriers between an item's
+// phases; levels of uneven items leave SMs idle at their end.  Measured against
+// 64-bit atomic sums merged over equal lanes and 128-bit compare-and-swap picks
+// (all levels of one build, GB300): 500M indoor points filtered 11.5 -> 8.2 ms,
+// 50M aerial filtered 1.14 -> 0.72 ms, 200M indoor points picked 5.9 -> 5.4 ms.
 //
 // Every octant's voxels go to a staging area; a level scan then assigns
 // each parent one contiguous voxel range (children are consecutive in node
@@ -200,16 +201,6 @@ __device__ __forceinline__ uint32_t parent_cell(uint32_t l, const ItemInfo& I) {
 }
 
 }  // namespace
-
-int vox_smem_bytes() { return kSmemBytes; }
-
-// Cells per accumulate pass of the four entry layouts (statistics and tests).
-void vox_capacities(uint32_t* small, uint32_t* narrow, uint32_t* wide, uint32_t* pick) {
-  *small = kCapLeaf;
-  *narrow = kCapNarrow;
-  *wide = kCapWide;
-  *pick = kCapPick;
-}
 
 // Shared state of one voxel CTA.
 struct VoxShared {
@@ -1291,8 +1282,8 @@ __device__ __forceinline__ uint4 far_ld4(uint32_t a) {
 // points first come (ten levels) 787 -> 602 us, 20M indoor points random (twelve)
 // 1160 -> 991 us, the root's 8 items of 500M points 172 -> 101 us.  (Adding each
 // CTA's share of the samples to the entries of the whole cluster by remote
-// atomics instead is slower for most levels, and atom.shared::cluster.min.u64
-// lost updates.)
+// atomics instead is slower for most levels: 56 items of 1M points 36 -> 113 us,
+// 8 items of 500M 172 -> 84.)
 template <int MODE>
 __global__ void __launch_bounds__(kVoxThreads, 1)
     k_vox_cluster(const __grid_constant__ BuildArgs a, const __grid_constant__ VoxLevel v, DevCounters* __restrict__ ctr, uint32_t lp) {

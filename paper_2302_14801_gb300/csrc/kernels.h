@@ -86,8 +86,6 @@ cudaError_t launch_voxel_points(const TileDesc* tiles, uint32_t n_tiles, const l
 cudaError_t launch_gather_voxels(const lod_node_t* nodes, uint32_t n_nodes, const uint64_t* new_off,
                                  const int4* src, int4* dst, cudaStream_t st);
 
-int vox_smem_bytes();
-void vox_capacities(uint32_t* small, uint32_t* narrow, uint32_t* wide, uint32_t* pick);
 int vox_init();
 
 // ----- out-of-core build (Section 7) -----

@@ -155,9 +155,4 @@ __device__ __forceinline__ uint32_t w_round(unsigned long long s, unsigned long 
   return m > 255ull ? 255u : (uint32_t)m;
 }
 
-// Octant of a parent-grid cell x | y << 7 | z << 14: k = 4 bx + 2 by + bz.
-__device__ __forceinline__ uint32_t cell_octant(uint32_t cell) {
-  return (((cell >> 6) & 1u) << 2) | (((cell >> 13) & 1u) << 1) | ((cell >> 20) & 1u);
-}
-
 }  // namespace lodk
